@@ -66,9 +66,7 @@ DEFAULT_WORKLOAD = "sphere-L9-const"
 # 4 x FFMA2 + 2 x FFMA + 2 x FADD2 + 2 x FMUL2 + FADD + FMUL (per-opcode thread counts:
 # the packed instructions are not in the FFMA/FADD class counters).
 KERNEL_COUNTERS = {
-    ("sphere-L9-const", "fp64"): dict(traffic=218932480 + 111733248, executed_flops=29402290440),
     ("sphere-L9-const", "fp32"): dict(traffic=177844224 + 104552192, executed_flops=47011848132),
-    ("sphere-L7-linear", "fp64"): dict(traffic=9516288 + 23808, executed_flops=2644445248),
     ("sphere-L7-linear", "fp32"): dict(traffic=9379072 + 512, executed_flops=3266600364),
 }
 COUNTER_SOURCE = "ncu --set full capture of one launch of this kernel on this workload"
@@ -234,20 +232,26 @@ class ClockSampler:
 # ------------------------------------------------------------ ALU peaks
 
 def measure_alu_peaks(dev, seconds=1.0, clk=None):
-    """FMA rate of the device's FP64 and FP32 pipes from the library's FMA-chain
-    probe (q2x_alu_peak_probe): a short calibration launch, then one launch
-    sized to about `seconds`, timed with CUDA events on the launching stream."""
+    """FMA rate of the device's FP64 and FP32 pipes and its integer multiply-add
+    rate from the library's chain probes (q2x_alu_peak_probe,
+    q2x_int_peak_probe): a short calibration launch, then one launch sized to
+    about `seconds`, timed with CUDA events on the launching stream."""
     import torch
-    from paper_2107_10942_gb300.q2x import alu_peak_probe
+    from paper_2107_10942_gb300.q2x import alu_peak_probe, int_peak_probe
     sink = torch.zeros(1, dtype=torch.float64, device=dev)
     stream = torch.cuda.current_stream()
     res = {}
-    for kind in ("dfma", "ffma", "ffma2"):
+    def probe(kind, iters):
+        if kind == "imad":
+            return int_peak_probe(iters, sink, stream)
+        return alu_peak_probe(kind, iters, sink, stream)
+
+    for kind in ("dfma", "ffma", "ffma2", "imad"):
         iters = 1024 if kind == "dfma" else 16384
         while True:
             a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
             a.record(stream)
-            alu_peak_probe(kind, iters, sink, stream)
+            probe(kind, iters)
             b.record(stream)
             b.synchronize()
             ms = a.elapsed_time(b)
@@ -258,14 +262,14 @@ def measure_alu_peaks(dev, seconds=1.0, clk=None):
         a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
         t0 = time.time()
         a.record(stream)
-        flops = alu_peak_probe(kind, iters, sink, stream)
+        flops = probe(kind, iters)
         b.record(stream)
         b.synchronize()
         t1 = time.time()
         ms = a.elapsed_time(b)
         if clk:
             clk.window("peak_" + kind, t0, t1)
-        res[kind] = {"tflops": flops / (ms * 1e-3) / 1e12, "ms": ms}
+        res[kind] = {"tmadds" if kind == "imad" else "tflops": flops / (ms * 1e-3) / 1e12, "ms": ms}
     return res
 
 
@@ -380,7 +384,7 @@ def main():
         dist.barrier()
     import paper_2107_10942_gb300 as q
     from paper_2107_10942_gb300.q2x import problem_to_device
-    from paper_2107_10942_gb300.roofline import element_flops
+    from paper_2107_10942_gb300.roofline import direction_madds, element_flops
 
     full = wl["gen"]()
     prob = full
@@ -411,7 +415,7 @@ def main():
         clk.start()
 
     peaks = measure_alu_peaks(dev, 1.0, clk)
-    peak64 = peaks["dfma"]["tflops"] * 1e12
+    peak64 = peaks["imad"]["tmadds"] * 1e12  # the FP64 leaf sums run on the integer pipe
     peak32 = max(peaks["ffma"]["tflops"], peaks["ffma2"]["tflops"]) * 1e12
 
     def step(plan, cs, cd):
@@ -562,7 +566,7 @@ def main():
         dist.all_reduce(t, op=dist.ReduceOp.SUM)
         total_moments = float(t.item())
     value = total_moments / (r64["ms"] * 1e-3)
-    flops_elem = element_flops("triangle", wl["density"], layers, P, point="order")  # FP64 kernel
+    madds_elem = direction_madds("triangle", wl["density"], layers, P)  # FP64 kernel: integer multiply-adds
     flops_elem32 = element_flops("triangle", wl["density"], layers, P)  # FP32 kernels: stencil on every level
 
     if rank != 0:
@@ -634,7 +638,7 @@ def main():
 
     k64 = KERNEL_COUNTERS.get((args.config, "fp64"), {})
     k32 = KERNEL_COUNTERS.get((args.config, "fp32"), {})
-    achieved64 = flops_elem * n_elem / (r64["kernel_ms"] * 1e-3)
+    achieved64 = madds_elem * n_elem / (r64["kernel_ms"] * 1e-3)
     achieved32 = flops_elem32 * n_elem / (r32["kernel_ms"] * 1e-3)
 
     def executed(kc, kernel_ms, peak):
@@ -654,16 +658,16 @@ def main():
                    "density": wl["density"], "layers": list(layers), "p": P, "n_elem": n_elem,
                    "moments_per_step": total_moments, "l2": "flushed between timed steps (256 MiB write)",
                    "parallelism": "leaf-sharded dp%d (no collective)" % world if world > 1 else "single GPU",
-                   "step": "one CUDA-graph replay: leaf-offset check, element kernel, fix-up of split leaves"},
-        "roofline": {"bound": "alu", "achieved": achieved64 / 1e12, "peak": peak64 / 1e12, "unit": "TFLOP/s",
-                     "frac": achieved64 / peak64, "traffic": k64.get("traffic"),
+                   "step": "one CUDA-graph replay: leaf-offset check, tile list, direction kernel, combine of split leaves"},
+        "roofline": {"bound": "integer multiply-add", "achieved": achieved64 / 1e12, "peak": peak64 / 1e12,
+                     "unit": "T 32x32+64-bit multiply-adds/s", "frac": achieved64 / peak64, "traffic": k64.get("traffic"),
                      "traffic_source": COUNTER_SOURCE if k64.get("traffic") else "not captured for this kernel",
-                     "kernel": "q2x_elem_kernel<double,%d,%s>" % (P, dname), "kernel_ms": r64["kernel_ms"],
-                     "flops_per_element": flops_elem, "flops_per_launch": flops_elem * n_elem,
+                     "kernel": "q2x_dir_kernel<%s> (directions, fixed point)" % dname, "kernel_ms": r64["kernel_ms"],
+                     "madds_per_element": madds_elem, "madds_per_launch": madds_elem * n_elem,
                      "algorithmic_bytes_per_launch": None,
                      "executed": executed(k64, r64["kernel_ms"], peak64),
-                     "peak_source": peak_src % ("DFMA", peaks["dfma"]["ms"] * 1e-3),
-                     "peak_fp64_fallback": "recipe: 152 SMs x 2 FP64 FMA/clk x 2 flops x 2.07 GHz = 1.26 TFLOP/s"},
+                     "peak_source": "measured in this run: q2x_int_peak_probe, %.2f s of 8 chains per thread on every "
+                                    "SM, CUDA events" % (peaks["imad"]["ms"] * 1e-3)},
         "fp32_mixed": {"value": total_moments / (r32["ms"] * 1e-3), "ms_per_step": r32["ms"],
                        "steps": r32["steps"], "speedup_vs_fp64": r64["ms"] / r32["ms"],
                        "roofline": {"bound": "alu", "achieved": achieved32 / 1e12, "peak": peak32 / 1e12,

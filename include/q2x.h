@@ -468,6 +468,9 @@ q2x_status q2x_leaf_reduce_weighted(q2x_plan_t plan, int64_t n_elem, int p, cons
  * Q2X_ERR_ARG for a bad kind, iters outside 1..2^40 or a NULL pointer. */
 typedef enum { Q2X_PEAK_DFMA = 0, Q2X_PEAK_FFMA = 1, Q2X_PEAK_FFMA2 = 2 } q2x_peak_kind;
 q2x_status q2x_alu_peak_probe(int kind, int64_t iters, double* sink, void* cuda_stream, double* flops);
+/* The same probe for the integer pipe that bounds the FP64 direction kernels:
+ * chains of 32 x 32 + 64-bit multiply-adds; *madds receives their number. */
+q2x_status q2x_int_peak_probe(int64_t iters, double* sink, void* cuda_stream, double* madds);
 
 #ifdef __cplusplus
 }

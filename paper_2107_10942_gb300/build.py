@@ -28,7 +28,7 @@ def _nvcc() -> str:
 
 def _flags():
     return ARCH + ["-O3", "-std=c++17", "-lineinfo", "-Xcompiler", "-fPIC", "-I", os.path.join(ROOT, "include"),
-                   "-I", CSRC]
+                   "-I", CSRC, "-I", OUT]
 
 
 def _stale(obj: str, deps) -> bool:
@@ -44,6 +44,12 @@ def build(force: bool = False, jobs: int | None = None, verbose: bool = False) -
     srcs = sorted(f for f in os.listdir(CSRC) if f.endswith(".cu"))
     headers = [os.path.join(CSRC, f) for f in os.listdir(CSRC) if f.endswith((".cuh", ".h"))]
     headers.append(os.path.join(ROOT, "include", "q2x.h"))
+    gen = os.path.join(HERE, "gen_directions.py")
+    table = os.path.join(OUT, "q2x_dirs_table.inc")
+    if force or _stale(table, [gen]):
+        subprocess.run([sys.executable, gen, table + ".tmp"], check=True)
+        os.replace(table + ".tmp", table)
+    headers.append(table)
     objs = []
     todo = []
     for s in srcs:

@@ -11,6 +11,7 @@
 
 #include "q2x.h"
 #include "q2x_batch.cuh"
+#include "q2x_dir.cuh"
 #include "q2x_kernels.cuh"
 #include "q2x_plan.h"
 
@@ -264,16 +265,101 @@ __global__ void leaf_reduce_weighted_kernel(const double* __restrict__ elem, int
 // Elements per leaf tile of the FP32-mixed single-layer path.
 constexpr int64_t kLeafTileElems = 256;
 
-// workspace of the leaf-tile path (after the per-leaf scales): the tile list,
+// workspace of the leaf-tile paths (after the per-leaf scales): the tile list,
 // the scans, and the partial rows of leaves of several tiles
-size_t leaf_tile_ws_bytes(int64_t n_elem, int64_t n_leaves, int np)
+size_t leaf_tile_ws_bytes(int64_t n_elem, int64_t n_leaves, int np, int64_t T, int layers = 1)
 {
     const int64_t nb = q2x::leaf_tile_blocks(n_leaves);
-    const int64_t mt = q2x::leaf_tile_max_tiles(n_leaves, n_elem, kLeafTileElems);
-    const int64_t ms = q2x::leaf_tile_max_slots(n_elem, kLeafTileElems);
+    const int64_t mt = q2x::leaf_tile_max_tiles(n_leaves, n_elem, T);
+    const int64_t ms = q2x::leaf_tile_max_slots(n_elem, T);
     return align_up(sizeof(q2x::BatchTile) * (size_t)mt, 256) + 2 * align_up(sizeof(int64_t) * (size_t)n_leaves, 256) +
            2 * align_up(sizeof(int64_t) * (size_t)nb, 256) + align_up(sizeof(int64_t) * (size_t)(n_leaves + 1), 256) +
-           256 + 256 + align_up(sizeof(double) * (size_t)ms * np, 256);
+           256 + 256 + layers * align_up(sizeof(double) * (size_t)ms * np, 256);
+}
+
+// the arrays of that workspace, from p on
+void leaf_tile_carve(unsigned char* p, int64_t n_elem, int64_t n_leaves, int np, int64_t T, int layers,
+                     q2x::LeafTileWork& w, double* partial[2])
+{
+    auto take = [&](size_t bytes) {
+        unsigned char* q = p;
+        p += align_up(bytes, 256);
+        return q;
+    };
+    const int64_t nb = q2x::leaf_tile_blocks(n_leaves);
+    w.max_tiles = q2x::leaf_tile_max_tiles(n_leaves, n_elem, T);
+    w.max_slots = q2x::leaf_tile_max_slots(n_elem, T);
+    w.n_elem = n_elem;
+    w.tiles = reinterpret_cast<q2x::BatchTile*>(take(sizeof(q2x::BatchTile) * (size_t)w.max_tiles));
+    w.tile_pre = reinterpret_cast<int64_t*>(take(sizeof(int64_t) * (size_t)n_leaves));
+    w.slot_pre = reinterpret_cast<int64_t*>(take(sizeof(int64_t) * (size_t)n_leaves));
+    w.block_tiles = reinterpret_cast<int64_t*>(take(sizeof(int64_t) * (size_t)nb));
+    w.block_slots = reinterpret_cast<int64_t*>(take(sizeof(int64_t) * (size_t)nb));
+    w.slot_off = reinterpret_cast<int64_t*>(take(sizeof(int64_t) * (size_t)(n_leaves + 1)));
+    w.n_tiles = reinterpret_cast<int64_t*>(take(sizeof(int64_t)));
+    w.counter = reinterpret_cast<unsigned long long*>(take(sizeof(unsigned long long)));
+    for (int l = 0; l < layers; ++l)
+        partial[l] = reinterpret_cast<double*>(take(sizeof(double) * (size_t)w.max_slots * np));
+}
+
+// FP64 leaf sums of one element set by the direction kernels
+q2x_status run_directions(q2x_plan_t plan, q2x::DirArgs& a, int kind, int dens, int combo, int T, int64_t n_elem,
+                          int64_t n_vert, const double* vxyz, const int32_t* idx, const double* sigma,
+                          int64_t n_leaves, const int64_t* leaf_off, const double* leaf_c, const int32_t* leaf_p,
+                          double* coef0, double* coef1, int accumulate)
+{
+    const int np = (plan->p_max + 1) * (plan->p_max + 1);
+    double* out[2] = {coef0 ? coef0 : coef1, coef0 ? coef1 : nullptr};
+    const int layers = out[1] ? 2 : 1;
+    q2x::LeafTileWork w;
+    double* partial[2] = {nullptr, nullptr};
+    leaf_tile_carve(static_cast<unsigned char*>(plan->ws), n_elem, n_leaves, np, T, layers, w, partial);
+    const int64_t nb = (n_leaves + 1 + 255) / 256;
+    check_leaf_off_kernel<<<(unsigned)nb, 256, 0, plan->stream>>>(leaf_off, n_leaves, n_elem, plan->d_err);
+    cudaError_t e = q2x::leaf_tiles_build(leaf_off, n_leaves, T, 0, 0, w, plan->stream);
+    if (e == cudaSuccess) e = cudaMemsetAsync(w.counter, 0, sizeof(unsigned long long), plan->stream);
+    if (e != cudaSuccess) return cuda_fail(plan, e, "leaf tile list");
+    a.kind = q2x::BatchKind{n_elem, n_vert, vxyz, vxyz + n_vert, vxyz + 2 * n_vert, idx, sigma};
+    a.n_leaves = n_leaves;
+    a.leaf_c = leaf_c;
+    a.leaf_p = leaf_p;
+    a.np = np;
+    a.norm = plan->norm;
+    a.accumulate = accumulate;
+    a.tiles = w.tiles;
+    a.n_tiles_dev = w.n_tiles;
+    a.counter = w.counter;
+    a.err = plan->d_err;
+    for (int l = 0; l < 2; ++l) {
+        a.partial[l] = partial[l];
+        a.coef[l] = out[l];
+    }
+    const q2x::DirFns& f = q2x::dir_fns()[combo];
+    int& occ = plan->dir_occ[combo];
+    if (occ == 0) {
+        e = f.occupancy(&occ, plan->p_max, T);
+        if (e != cudaSuccess) return cuda_fail(plan, e, "direction kernel occupancy query");
+        if (occ <= 0) return fail(plan, Q2X_ERR_CUDA, "direction kernel does not fit on the device");
+    }
+    cudaEvent_t ev0 = nullptr, ev1 = nullptr;
+    if (plan->timing) {
+        q2x_status st = take_event(plan, &ev0);
+        if (st == Q2X_OK) st = take_event(plan, &ev1);
+        if (st != Q2X_OK) return st;
+        cudaEventRecord(ev0, plan->stream);
+    }
+    const int64_t grid = std::min<int64_t>((int64_t)occ * plan->num_sms, w.max_tiles);
+    e = f.launch(a, T, (int)grid, plan->stream);
+    if (e != cudaSuccess) return cuda_fail(plan, e, "direction kernel launch");
+    if (plan->timing) {
+        cudaEventRecord(ev1, plan->stream);
+        plan->ev_pending.emplace_back(ev0, ev1);
+    }
+    for (int l = 0; l < layers && e == cudaSuccess; ++l)
+        e = q2x::leaf_tiles_combine(partial[l], w.slot_off, leaf_off, np, n_leaves, out[l], accumulate, plan->stream);
+    if (e != cudaSuccess) return cuda_fail(plan, e, "leaf tile combine");
+    plan->launches += 5 + layers;
+    return Q2X_OK;
 }
 
 q2x_status run_elements(q2x_plan_t plan, int kind, int dens, int64_t n_elem, int64_t n_vert,
@@ -344,7 +430,28 @@ q2x_status run_elements(q2x_plan_t plan, int kind, int dens, int64_t n_elem, int
     // (its workspace bound assumes every tile needs a partial row: beyond
     // 8 GiB the element kernel, whose workspace is per warp range, runs)
     const bool tiles = prec == 1 && leaf_off && !vec && coef0 && !(kind == q2x::KIND_TRI && coef1) &&
-                       n_leaves < ((int64_t)1 << 31) && leaf_tile_ws_bytes(n_elem, n_leaves, np) <= ((size_t)8 << 30);
+                       n_leaves < ((int64_t)1 << 31) &&
+                       leaf_tile_ws_bytes(n_elem, n_leaves, np, kLeafTileElems) <= ((size_t)8 << 30);
+    // FP64 in leaf mode: the same tile list through the direction kernels
+    // (q2x_dir.cuh), within the same workspace bound
+    const bool dirs = prec == 0 && leaf_off && !vec && n_leaves < ((int64_t)1 << 31);
+    q2x::DirArgs da{};
+    int dir_T = 0;
+    const int dir_layers = (coef0 ? 1 : 0) + (dbl ? 1 : 0);
+    size_t dir_bytes = 0;
+    if (dirs) {
+        da.p_max = plan->p_max;
+        e = q2x::dir_setup(da, kind, dens);
+        dir_T = q2x::dir_tile_elems(plan->p_max);
+        if (e != cudaSuccess) return cuda_fail(plan, e, "direction tables");
+        dir_bytes = leaf_tile_ws_bytes(n_elem, n_leaves, np, dir_T, dir_layers);
+    }
+    if (dirs && dir_bytes <= ((size_t)8 << 30)) {
+        q2x_status st = ensure_ws(plan, dir_bytes);
+        if (st != Q2X_OK) return st;
+        return run_directions(plan, da, kind, dens, combo, dir_T, n_elem, n_vert, vxyz, idx, sigma, n_leaves, leaf_off,
+                              leaf_c, leaf_p, coef0, dbl ? coef1 : nullptr, accumulate);
+    }
     const int64_t resident_warps = (int64_t)occ * wpc * plan->num_sms;
     // one range per resident warp (ranges need not be multiples of 32: rounds
     // are formed per leaf inside the kernel), at least one full round each
@@ -357,7 +464,7 @@ q2x_status run_elements(q2x_plan_t plan, int kind, int dens, int64_t n_elem, int
     const size_t slot_bytes = tiles ? 0 : align_up(sizeof(double) * (size_t)n_ranges * 2 * nacc * np, 256);  // FP64 partials
     const size_t rho_bytes = need_rho ? align_up(sizeof(double) * (size_t)n_leaves, 256) : 0;
     const size_t bits_bytes = need_rho ? align_up(sizeof(int) * (size_t)n_leaves, 256) : 0;
-    const size_t tile_bytes = tiles ? leaf_tile_ws_bytes(n_elem, n_leaves, np) : 0;
+    const size_t tile_bytes = tiles ? leaf_tile_ws_bytes(n_elem, n_leaves, np, kLeafTileElems) : 0;
     q2x_status st = ensure_ws(plan, slot_bytes + rho_bytes + bits_bytes + tile_bytes);
     if (st != Q2X_OK) return st;
     unsigned char* ws = static_cast<unsigned char*>(plan->ws);
@@ -380,28 +487,9 @@ q2x_status run_elements(q2x_plan_t plan, int kind, int dens, int64_t n_elem, int
     }
 
     if (tiles) {
-        unsigned char* p = ws + slot_bytes + rho_bytes + bits_bytes;
-        auto take = [&](size_t bytes) {
-            unsigned char* q = p;
-            p += align_up(bytes, 256);
-            return q;
-        };
-        const int64_t nb = q2x::leaf_tile_blocks(n_leaves);
-        const int64_t mt = q2x::leaf_tile_max_tiles(n_leaves, n_elem, kLeafTileElems);
-        const int64_t ms = q2x::leaf_tile_max_slots(n_elem, kLeafTileElems);
         q2x::LeafTileWork w;
-        w.tiles = reinterpret_cast<q2x::BatchTile*>(take(sizeof(q2x::BatchTile) * (size_t)mt));
-        w.tile_pre = reinterpret_cast<int64_t*>(take(sizeof(int64_t) * (size_t)n_leaves));
-        w.slot_pre = reinterpret_cast<int64_t*>(take(sizeof(int64_t) * (size_t)n_leaves));
-        w.block_tiles = reinterpret_cast<int64_t*>(take(sizeof(int64_t) * (size_t)nb));
-        w.block_slots = reinterpret_cast<int64_t*>(take(sizeof(int64_t) * (size_t)nb));
-        w.slot_off = reinterpret_cast<int64_t*>(take(sizeof(int64_t) * (size_t)(n_leaves + 1)));
-        w.n_tiles = reinterpret_cast<int64_t*>(take(sizeof(int64_t)));
-        w.counter = reinterpret_cast<unsigned long long*>(take(sizeof(unsigned long long)));
-        double* partial = reinterpret_cast<double*>(take(sizeof(double) * (size_t)ms * np));
-        w.max_tiles = mt;
-        w.max_slots = ms;
-        w.n_elem = n_elem;
+        double* partial[2] = {nullptr, nullptr};
+        leaf_tile_carve(ws + slot_bytes + rho_bytes + bits_bytes, n_elem, n_leaves, np, kLeafTileElems, 1, w, partial);
         const int tcombo = (kind == q2x::KIND_SEG) ? 0 : (kind == q2x::KIND_TET) ? 3 : (dens == Q2X_DENSITY_LINEAR ? 2 : 1);
         const q2x::BatchGroupFns& f = q2x::batch_group_table_f32()[tcombo * 5 + bin];
         int& tocc = plan->tile_occ[tcombo][bin];
@@ -431,7 +519,7 @@ q2x_status run_elements(q2x_plan_t plan, int kind, int dens, int64_t n_elem, int
         b.tiles = w.tiles;
         b.n_tiles = 0;
         b.counter = w.counter;
-        b.partial = partial;
+        b.partial = partial[0];
         b.err = plan->d_err;
         b.coef = coef0;
         b.accumulate = accumulate;
@@ -449,7 +537,7 @@ q2x_status run_elements(q2x_plan_t plan, int kind, int dens, int64_t n_elem, int
             cudaEventRecord(ev1, plan->stream);
             plan->ev_pending.emplace_back(ev0, ev1);
         }
-        e = q2x::leaf_tiles_combine(partial, w.slot_off, leaf_off, np, n_leaves, coef0, accumulate, plan->stream);
+        e = q2x::leaf_tiles_combine(partial[0], w.slot_off, leaf_off, np, n_leaves, coef0, accumulate, plan->stream);
         if (e != cudaSuccess) return cuda_fail(plan, e, "leaf tile combine");
         plan->launches += 5;
         return Q2X_OK;
@@ -653,7 +741,8 @@ q2x_status q2x_reserve(q2x_plan_t plan, int64_t n_elem, int64_t n_leaves)
     // worst case: one range per 32 elements; FP64 partials in both precisions
     const int64_t n_ranges = (n_elem + 31) / 32;
     const size_t elem = align_up(sizeof(double) * (size_t)n_ranges * 2 * 3 * np, 256);
-    size_t tile = plan->prec == 1 ? leaf_tile_ws_bytes(n_elem, n_leaves, np) : 0;
+    size_t tile = plan->prec == 1 ? leaf_tile_ws_bytes(n_elem, n_leaves, np, kLeafTileElems)
+                                  : leaf_tile_ws_bytes(n_elem, n_leaves, np, q2x::dir_tile_elems(plan->p_max), 2);
     if (tile > ((size_t)8 << 30)) tile = 0;  // such calls run the element kernel
     const size_t bytes = std::max(elem, tile) + align_up(sizeof(double) * (size_t)n_leaves, 256) +
                          align_up(sizeof(int) * (size_t)n_leaves, 256);

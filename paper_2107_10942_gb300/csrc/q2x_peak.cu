@@ -1,7 +1,7 @@
 // q2x_peak.cu -- ALU peak probes (declared in include/q2x.h).
 //
 // A measurement aid for the roofline of the element kernels, which are bound
-// by the FP64 or FP32 FMA pipes: one launch of independent FMA chains on every
+// by the FP64, FP32 or integer pipes: one launch of independent chains on every
 // SM of the device, from which the caller forms flops / (CUDA-event time).
 // Each thread runs CHAINS independent chains x <- x * a + b (|a| < 1, so the
 // values stay near b / (1 - a) and never overflow or become denormal); the
@@ -86,7 +86,51 @@ __global__ void __launch_bounds__(THREADS) peak_ffma2_kernel(int64_t iters, doub
     if (s == -1.f) sink[0] = (double)s;
 }
 
+// 32 x 32 + 64-bit integer multiply-adds, operands taken from the running sums
+__global__ void __launch_bounds__(THREADS) peak_imad_kernel(int64_t iters, double* sink)
+{
+    long long x[CHAINS];
+#pragma unroll
+    for (int j = 0; j < CHAINS; ++j) x[j] = (long long)(threadIdx.x + 1) * 0x12345678abcdefll + j;
+#pragma unroll 1
+    for (int64_t it = 0; it < iters; it += UNROLL) {
+#pragma unroll
+        for (int u = 0; u < UNROLL; ++u)
+#pragma unroll
+            for (int j = 0; j < CHAINS; ++j) {
+                const int a = (int)x[(j + 1) % CHAINS], b = (int)(x[(j + 2) % CHAINS] >> 32);
+                long long m;
+                asm("mul.wide.s32 %0, %1, %2;" : "=l"(m) : "r"(a), "r"(b));
+                asm volatile("add.s64 %0, %0, %1;" : "+l"(x[j]) : "l"(m));
+            }
+    }
+    long long s = 0;
+#pragma unroll
+    for (int j = 0; j < CHAINS; ++j) s ^= x[j];
+    if (s == 0x7fffffffffffffffll) sink[0] = (double)s;
+}
+
 }  // namespace
+
+extern "C" q2x_status q2x_int_peak_probe(int64_t iters, double* sink, void* cuda_stream, double* madds)
+{
+    if (iters <= 0 || iters > ((int64_t)1 << 40)) return q2x_fail(nullptr, Q2X_ERR_ARG, "iters out of range");
+    if (!sink || !madds) return q2x_fail(nullptr, Q2X_ERR_ARG, "sink and madds must be non-NULL");
+    int dev = 0, sms = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e != cudaSuccess) {
+        cudaGetLastError();
+        return q2x_cuda_fail(nullptr, e, "device query");
+    }
+    iters = (iters + UNROLL - 1) / UNROLL * UNROLL;
+    const int grid = sms * CTAS_PER_SM;
+    peak_imad_kernel<<<grid, THREADS, 0, static_cast<cudaStream_t>(cuda_stream)>>>(iters, sink);
+    *madds = (double)grid * THREADS * CHAINS * (double)iters;
+    e = cudaGetLastError();
+    if (e != cudaSuccess) return q2x_cuda_fail(nullptr, e, "probe launch");
+    return Q2X_OK;
+}
 
 extern "C" q2x_status q2x_alu_peak_probe(int kind, int64_t iters, double* sink, void* cuda_stream,
                                          double* flops)

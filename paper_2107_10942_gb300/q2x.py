@@ -493,6 +493,17 @@ def alu_peak_probe(kind: str, iters: int, sink, stream=None) -> float:
     return float(flops.value)
 
 
+def int_peak_probe(iters: int, sink, stream=None) -> float:
+    """alu_peak_probe for the integer pipe (q2x_int_peak_probe); returns the
+    32 x 32 + 64-bit multiply-adds the launch performs."""
+    _need(sink, torch.float64, "sink")
+    if stream is None:
+        stream = torch.cuda.current_stream()
+    madds = ctypes.c_double(0.0)
+    check(lib().q2x_int_peak_probe(int(iters), _ptr(sink), ctypes.c_void_p(stream.cuda_stream), ctypes.byref(madds)))
+    return float(madds.value)
+
+
 def problem_to_device(prob: dict, device="cuda") -> dict:
     """Copy a workloads-style problem dict (numpy arrays) to device tensors."""
     out = {}

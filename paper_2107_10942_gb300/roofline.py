@@ -87,3 +87,16 @@ def vjp_flops(p: int = 12) -> int:
     rows (8 adds each)."""
     entries = sum(n + 1 for n in range(p + 1))
     return 7 * level_flops(p) + 10 * 4 * entries + 3 * 8 * entries
+
+
+def direction_madds(kind: str, density: str = "const", layers=("single",), p: int = 12) -> int:
+    """32 x 32 + 64-bit integer multiply-adds per element of the FP64 direction
+    kernels: a real product of two 62-bit numbers is three; per direction (p +
+    1 of them) and degree 1..p a complex product (12) per level and for the
+    double layer, for linear density also the three real multiples of complex
+    values (18) and (n + 1) q (2); per direction the dot products a . y of the
+    vertices and the normal (18 each)."""
+    nv = {"segment": 2, "triangle": 3, "tetra": 4}[kind]
+    dbl = "double" in layers
+    step = 12 * (nv if density == "const" else 5) + (12 if dbl else 0) + (20 if density == "linear" else 0)
+    return (p + 1) * (p * step + 18 * (nv + (1 if dbl else 0)))

@@ -1,0 +1,126 @@
+"""The FP64 leaf sums by directions (csrc/q2x_dir.cuh) at the sizes where their
+tiling and number format could go wrong: tiles that are just full, just over
+and nearly empty, every kind and layer at degrees between the tested bins,
+coordinates in other units, and very uneven weights.  Reference: the same
+library's per-element rows (the FP64 row kernel, another algorithm), summed in
+leaves by q2x_leaf_reduce.
+
+Tolerance: both paths round each element's moments to a few units of 2^-53 of
+its own scale, and a leaf of K elements sums K of them; with K <= 700 and the
+scaled norm of _helpers (degree n over rho^n) 1e-12 is the suite's FP64 bound."""
+import numpy as np
+import pytest
+from _helpers import norm_err, random_problem
+
+pytestmark = pytest.mark.gpu
+KINDS = [("segment", "const"), ("triangle", "const"), ("triangle", "linear"), ("tetra", "const")]
+
+
+@pytest.fixture(scope="module")
+def q2x():
+    import paper_2107_10942_gb300 as q
+    return q
+
+
+def call(plan, prob, off, c, rho, lp, layers):
+    import torch
+    d = {k: torch.from_numpy(np.ascontiguousarray(v)).cuda() for k, v in prob.items() if hasattr(v, "dtype")}
+    t = [None if x is None else torch.from_numpy(np.ascontiguousarray(x)).cuda() for x in (off, c, rho, lp)]
+    args = (d["vxyz"], d["idx"], d["sigma"], *t)
+    if prob["kind"] == "segment":
+        return [plan.segments(*args)]
+    if prob["kind"] == "tetra":
+        return [plan.tetra(*args)]
+    return list(plan.triangles(*args, density=prob["density"], single=layers[0], double=layers[1]))
+
+
+def both(q2x, prob, p, layers, rho=True, norm="coeff"):
+    """(leaf sums, per-element rows summed in leaves), each a list over the layers."""
+    import torch
+    plan = q2x.Plan(p, norm=norm)
+    off = prob["leaf_off"]
+    leaf_of = np.repeat(np.arange(len(off) - 1), np.diff(off))
+    got = call(plan, prob, off, prob["leaf_c"], prob["leaf_rho"] if rho else None, prob["leaf_p"], layers)
+    rows = call(plan, prob, None, prob["leaf_c"][:, leaf_of], prob["leaf_rho"][leaf_of] if rho else None,
+                prob["leaf_p"][leaf_of], layers)
+    off_d = torch.from_numpy(off).cuda()
+    ref = [None if r is None else plan.leaf_reduce(r, p, off_d) for r in rows]
+    plan.sync()
+    return got, ref
+
+
+def check(prob, p, got, ref):
+    for layer, (g, r) in enumerate(zip(got, ref)):
+        if r is not None:
+            assert norm_err(g.cpu().numpy(), r.cpu().numpy(), p, prob["leaf_rho"], layer) <= 1e-12
+
+
+@pytest.mark.parametrize("kind,density", KINDS)
+@pytest.mark.parametrize("p", [0, 1, 2, 5, 11, 13, 15, 18, 20])
+def test_tile_edges(q2x, kind, density, p):
+    groups = 256 // (p + 1)
+    full = min(8 * groups, 256)
+    sizes = [1, groups - 1, groups, groups + 1, full - 1, full, 0, full + 1, min(2 * full + 1, 600), 2, 7, 8, 9, 33]
+    prob = random_problem(kind, sizes, seed=p + 50, p=p, density=density)
+    layers = (True, kind == "triangle")
+    check(prob, p, *both(q2x, prob, p, layers))
+
+
+@pytest.mark.parametrize("layers", [(True, False), (False, True), (True, True)])
+@pytest.mark.parametrize("density", ["const", "linear"])
+def test_layers_and_ragged_degrees(q2x, layers, density):
+    p, sizes = 17, [5, 120, 121, 1, 64]
+    prob = random_problem("triangle", sizes, seed=3, p=p, density=density, leaf_p=[17, 3, 16, 0, 9])
+    check(prob, p, *both(q2x, prob, p, layers, norm="moment"))
+
+
+@pytest.mark.parametrize("unit", [1e-140, 1e-30, 3.7, 1e25, 1e90])
+@pytest.mark.parametrize("kind,density", KINDS)
+def test_units(q2x, kind, density, unit):
+    """Coordinates in another unit scale degree n of a kind of dimension d by
+    unit^(n + d) (single layer); p = 2 keeps that inside FP64 at these units."""
+    p = 2
+    prob = random_problem(kind, [9, 40, 3], seed=8, p=p, density=density)
+    base, _ = both(q2x, prob, p, (True, False))
+    for k in ("vxyz", "leaf_c", "leaf_rho"):
+        prob[k] = prob[k] * unit
+    got = both(q2x, prob, p, (True, False), rho=False)[0][0].cpu().numpy()
+    dim = {"segment": 1, "triangle": 2, "tetra": 3}[kind]
+    scale = np.concatenate([np.full(2 * n + 1, float(n + dim)) for n in range(p + 1)])
+    with np.errstate(over="ignore", under="ignore"):
+        want = base[0].cpu().numpy() * unit ** scale
+    ok = (np.abs(want) > 1e-290) & np.isfinite(want)
+    # the scaled coordinates themselves are rounded: up to (p + 1) units of 2^-53 of the leaf's largest
+    for n in range(p + 1):
+        cols = slice(n * n, (n + 1) ** 2)
+        big = np.max(np.abs(np.where(ok, want, 0.0))[:, cols], axis=1, keepdims=True)
+        diff = np.abs(np.where(ok, got, 0.0) - np.where(ok, want, 0.0))[:, cols]
+        assert np.all(diff <= 1e-12 * big + 1e-290)
+    assert np.array_equal(np.isinf(got), np.isinf(want))  # beyond FP64 in both
+
+
+def test_uneven_weights(q2x):
+    """A heavy element beside light ones, and elements of no weight far out: the
+    sums stay relative to the leaf's largest term."""
+    p = 12
+    prob = random_problem("triangle", [50, 50], seed=4, p=p)
+    prob["sigma"][:25] *= 1e-9
+    prob["sigma"][60:] = 0.0
+    check(prob, p, *both(q2x, prob, p, (True, True)))
+
+
+def test_accumulate_and_repeat(q2x):
+    """Accumulation into leaves of one and of several tiles, and bit equality of repeated calls."""
+    import torch
+    p = 9
+    prob = random_problem("triangle", [0, 3, 700, 90], seed=6, p=p)
+    plan = q2x.Plan(p)
+    d = {k: torch.from_numpy(np.ascontiguousarray(v)).cuda() for k, v in prob.items() if hasattr(v, "dtype")}
+    args = (d["vxyz"], d["idx"], d["sigma"], d["leaf_off"], d["leaf_c"], d["leaf_rho"], d["leaf_p"])
+    one, _ = plan.triangles(*args)
+    again, _ = plan.triangles(*args)
+    assert torch.equal(one, again)
+    base = torch.rand_like(one)
+    acc = base.clone()
+    plan.triangles(*args, coef_single=acc, accumulate=True)
+    assert torch.equal(acc, base + one)
