@@ -279,7 +279,7 @@ size_t leaf_tile_ws_bytes(int64_t n_elem, int64_t n_leaves, int np, int64_t T, i
 
 // the arrays of that workspace, from p on
 void leaf_tile_carve(unsigned char* p, int64_t n_elem, int64_t n_leaves, int np, int64_t T, int layers,
-                     q2x::LeafTileWork& w, double* partial[2])
+                     q2x::LeafTileWork& w, double** partial)
 {
     auto take = [&](size_t bytes) {
         unsigned char* q = p;
@@ -306,13 +306,17 @@ void leaf_tile_carve(unsigned char* p, int64_t n_elem, int64_t n_leaves, int np,
 q2x_status run_directions(q2x_plan_t plan, q2x::DirArgs& a, int kind, int dens, int combo, int T, int64_t n_elem,
                           int64_t n_vert, const double* vxyz, const int32_t* idx, const double* sigma,
                           int64_t n_leaves, const int64_t* leaf_off, const double* leaf_c, const int32_t* leaf_p,
-                          double* coef0, double* coef1, int accumulate)
+                          double* coef0, double* coef1, int accumulate, const double* wvec, double* coef2)
 {
     const int np = (plan->p_max + 1) * (plan->p_max + 1);
-    double* out[2] = {coef0 ? coef0 : coef1, coef0 ? coef1 : nullptr};
-    const int layers = out[1] ? 2 : 1;
+    double* out[3] = {coef0, coef1, coef2};  // a vector density's components, NULL = not wanted
+    if (!wvec && !coef0) {
+        out[0] = coef1;
+        out[1] = nullptr;
+    }
+    const int layers = wvec ? 3 : out[1] ? 2 : 1;
     q2x::LeafTileWork w;
-    double* partial[2] = {nullptr, nullptr};
+    double* partial[3] = {nullptr, nullptr, nullptr};
     leaf_tile_carve(static_cast<unsigned char*>(plan->ws), n_elem, n_leaves, np, T, layers, w, partial);
     const int64_t nb = (n_leaves + 1 + 255) / 256;
     check_leaf_off_kernel<<<(unsigned)nb, 256, 0, plan->stream>>>(leaf_off, n_leaves, n_elem, plan->d_err);
@@ -330,7 +334,8 @@ q2x_status run_directions(q2x_plan_t plan, q2x::DirArgs& a, int kind, int dens, 
     a.n_tiles_dev = w.n_tiles;
     a.counter = w.counter;
     a.err = plan->d_err;
-    for (int l = 0; l < 2; ++l) {
+    a.wvec = wvec;
+    for (int l = 0; l < 3; ++l) {
         a.partial[l] = partial[l];
         a.coef[l] = out[l];
     }
@@ -356,7 +361,8 @@ q2x_status run_directions(q2x_plan_t plan, q2x::DirArgs& a, int kind, int dens, 
         plan->ev_pending.emplace_back(ev0, ev1);
     }
     for (int l = 0; l < layers && e == cudaSuccess; ++l)
-        e = q2x::leaf_tiles_combine(partial[l], w.slot_off, leaf_off, np, n_leaves, out[l], accumulate, plan->stream);
+        if (out[l])
+            e = q2x::leaf_tiles_combine(partial[l], w.slot_off, leaf_off, np, n_leaves, out[l], accumulate, plan->stream);
     if (e != cudaSuccess) return cuda_fail(plan, e, "leaf tile combine");
     plan->launches += 5 + layers;
     return Q2X_OK;
@@ -434,15 +440,15 @@ q2x_status run_elements(q2x_plan_t plan, int kind, int dens, int64_t n_elem, int
                        leaf_tile_ws_bytes(n_elem, n_leaves, np, kLeafTileElems) <= ((size_t)8 << 30);
     // FP64 in leaf mode: the same tile list through the direction kernels
     // (q2x_dir.cuh), within the same workspace bound
-    const bool dirs = prec == 0 && leaf_off && !vec && n_leaves < ((int64_t)1 << 31);
+    const bool dirs = prec == 0 && leaf_off && n_leaves < ((int64_t)1 << 31);
     q2x::DirArgs da{};
     int dir_T = 0;
-    const int dir_layers = (coef0 ? 1 : 0) + (dbl ? 1 : 0);
+    const int dir_layers = vec ? 3 : (coef0 ? 1 : 0) + (dbl ? 1 : 0);
     size_t dir_bytes = 0;
     if (dirs) {
         da.p_max = plan->p_max;
-        e = q2x::dir_setup(da, kind, dens);
-        dir_T = q2x::dir_tile_elems(plan->p_max);
+        e = q2x::dir_setup(da, kind, dens, vec);
+        dir_T = q2x::dir_tile_elems(plan->p_max, vec);
         if (e != cudaSuccess) return cuda_fail(plan, e, "direction tables");
         dir_bytes = leaf_tile_ws_bytes(n_elem, n_leaves, np, dir_T, dir_layers);
     }
@@ -450,7 +456,7 @@ q2x_status run_elements(q2x_plan_t plan, int kind, int dens, int64_t n_elem, int
         q2x_status st = ensure_ws(plan, dir_bytes);
         if (st != Q2X_OK) return st;
         return run_directions(plan, da, kind, dens, combo, dir_T, n_elem, n_vert, vxyz, idx, sigma, n_leaves, leaf_off,
-                              leaf_c, leaf_p, coef0, dbl ? coef1 : nullptr, accumulate);
+                              leaf_c, leaf_p, coef0, dbl || vec ? coef1 : nullptr, accumulate, wvec, coef2);
     }
     const int64_t resident_warps = (int64_t)occ * wpc * plan->num_sms;
     // one range per resident warp (ranges need not be multiples of 32: rounds
@@ -742,7 +748,10 @@ q2x_status q2x_reserve(q2x_plan_t plan, int64_t n_elem, int64_t n_leaves)
     const int64_t n_ranges = (n_elem + 31) / 32;
     const size_t elem = align_up(sizeof(double) * (size_t)n_ranges * 2 * 3 * np, 256);
     size_t tile = plan->prec == 1 ? leaf_tile_ws_bytes(n_elem, n_leaves, np, kLeafTileElems)
-                                  : leaf_tile_ws_bytes(n_elem, n_leaves, np, q2x::dir_tile_elems(plan->p_max), 2);
+                                  : std::max(leaf_tile_ws_bytes(n_elem, n_leaves, np,
+                                                                q2x::dir_tile_elems(plan->p_max, false), 2),
+                                             leaf_tile_ws_bytes(n_elem, n_leaves, np,
+                                                                q2x::dir_tile_elems(plan->p_max, true), 3));
     if (tile > ((size_t)8 << 30)) tile = 0;  // such calls run the element kernel
     const size_t bytes = std::max(elem, tile) + align_up(sizeof(double) * (size_t)n_leaves, 256) +
                          align_up(sizeof(int) * (size_t)n_leaves, 256);

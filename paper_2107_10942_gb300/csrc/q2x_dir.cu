@@ -13,7 +13,7 @@ namespace {
 template <int KIND, int DENS, int OUTS>
 cudaError_t dir_attr(int p, int T, size_t* smem)
 {
-    *smem = DirCfg<KIND, DENS, OUTS>::smem(p, T, dir_threads(p));
+    *smem = DirCfg<KIND, DENS, OUTS>::smem(p, T, dir_threads(p, (OUTS & 4) != 0));
     return cudaFuncSetAttribute(q2x_dir_kernel<KIND, DENS, OUTS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 (int)*smem);
 }
@@ -24,7 +24,7 @@ cudaError_t dir_launch(const DirArgs& a, int T, int grid, cudaStream_t st)
     size_t smem;
     cudaError_t e = dir_attr<KIND, DENS, OUTS>(a.p_max, T, &smem);
     if (e != cudaSuccess) return e;
-    q2x_dir_kernel<KIND, DENS, OUTS><<<grid, dir_threads(a.p_max), smem, st>>>(a, T);
+    q2x_dir_kernel<KIND, DENS, OUTS><<<grid, dir_threads(a.p_max, (OUTS & 4) != 0), smem, st>>>(a, T);
     return cudaGetLastError();
 }
 
@@ -35,7 +35,7 @@ cudaError_t dir_occupancy(int* blocks, int p, int T)
     cudaError_t e = dir_attr<KIND, DENS, OUTS>(p, T, &smem);
     if (e != cudaSuccess) return e;
     return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks, q2x_dir_kernel<KIND, DENS, OUTS>,
-                                                         dir_threads(p), smem);
+                                                         dir_threads(p, (OUTS & 4) != 0), smem);
 }
 
 #define Q2X_DIR_FNS(K, D, O) {&dir_launch<K, D, O>, &dir_occupancy<K, D, O>}
@@ -45,19 +45,21 @@ cudaError_t dir_occupancy(int* blocks, int p, int T)
 // 256 threads, 17 directions: 255 at work at p = 16.  Smaller CTAs overlap
 // their phases better but map twice as many tiles to coefficients (level-9
 // sphere, p = 16: 11.4 ms with 256 threads, 11.6 with 128, 12.6 with 160).
-int dir_threads(int) { return 256; }
+// The three sums of a vector density take three times the shared memory: 128.
+int dir_threads(int, bool vec) { return vec ? 128 : 256; }
 
 const DirFns* dir_fns()
 {
-    static const DirFns f[8] = {
+    static const DirFns f[9] = {
         Q2X_DIR_FNS(KIND_SEG, DENS_CONST, 1),  Q2X_DIR_FNS(KIND_TRI, DENS_CONST, 1),
         Q2X_DIR_FNS(KIND_TRI, DENS_CONST, 2),  Q2X_DIR_FNS(KIND_TRI, DENS_CONST, 3),
         Q2X_DIR_FNS(KIND_TRI, DENS_LINEAR, 1), Q2X_DIR_FNS(KIND_TRI, DENS_LINEAR, 2),
-        Q2X_DIR_FNS(KIND_TRI, DENS_LINEAR, 3), Q2X_DIR_FNS(KIND_TET, DENS_CONST, 1)};
+        Q2X_DIR_FNS(KIND_TRI, DENS_LINEAR, 3), Q2X_DIR_FNS(KIND_TET, DENS_CONST, 1),
+        Q2X_DIR_FNS(KIND_SEG, DENS_CONST, 4)};
     return f;
 }
 
-cudaError_t dir_setup(DirArgs& a, int kind, int dens)
+cudaError_t dir_setup(DirArgs& a, int kind, int dens, bool vector)
 {
     const int p = a.p_max;
     void *vec, *inv, *eighth, *pw, *col;
@@ -73,7 +75,7 @@ cudaError_t dir_setup(DirArgs& a, int kind, int dens)
     a.pw = static_cast<const double*>(pw);
     a.col = static_cast<const double*>(col);
     a.J = p + 1;
-    a.G = dir_threads(p) / a.J;
+    a.G = dir_threads(p, vector) / a.J;
     a.rnd = (long long)((1ull << 63) + (1ull << 31));
     // Bound of a level's value over the seed's (|u| < 1): the dimension's
     // binomial, for linear density (n+1)(n+2)(n+3)/2 of a half.  Seeds start at

@@ -204,8 +204,9 @@ struct DirArgs {
     const BatchTile* tiles;
     const int64_t* n_tiles_dev;
     unsigned long long* counter;
-    double* partial[2];
-    double* coef[2];
+    const double* wvec;  // vector density: SoA 3 x n_elem components per element
+    double* partial[3];
+    double* coef[3];
     unsigned* err;
 };
 
@@ -218,13 +219,15 @@ struct DirCfg {
     static constexpr int NV = KIND + 2;
     static constexpr bool LIN = KIND == KIND_TRI && DENS == DENS_LINEAR;
     static constexpr bool DBL = KIND == KIND_TRI && (OUTS & 2) != 0;
-    static constexpr bool SGL = (OUTS & 1) != 0;
+    // a vector density: unit-density values, three weighted sums
+    static constexpr bool VEC = (OUTS & 4) != 0;
+    static constexpr bool SGL = (OUTS & 1) != 0 || VEC;
     static constexpr int NL = KIND + 2 + (LIN ? 2 : 0);  // q, p | j, i | b, a; linear: q, j, E, i, Iw
     // what the stored values of level k carry, in units of 2^32 (mul2)
     __host__ __device__ static constexpr int bias(int k) { return LIN && k >= 2 ? k : k + 1; }
-    static constexpr int LAYERS = (SGL ? 1 : 0) + (DBL ? 1 : 0);
+    static constexpr int LAYERS = VEC ? 3 : (SGL ? 1 : 0) + (DBL ? 1 : 0);
     // 8-byte words of a record: vertices, then the normal, then the densities, then the seed
-    static constexpr int R_NRM = 3 * NV, R_DENS = R_NRM + (DBL ? 3 : 0), R_SEED = R_DENS + (LIN ? 3 : 0);
+    static constexpr int R_NRM = 3 * NV, R_DENS = R_NRM + (DBL ? 3 : 0), R_SEED = R_DENS + (LIN || VEC ? 3 : 0);
     static constexpr int REC = R_SEED + 1;
     __host__ __device__ static constexpr size_t rec_bytes(int p, int T)
     {
@@ -246,7 +249,7 @@ __global__ void __launch_bounds__(DIR_MAX_NT, 2) q2x_dir_kernel(const DirArgs a,
     using D = DirCfg<KIND, DENS, OUTS>;
     constexpr int NV = D::NV;
     constexpr int NL = D::NL;
-    constexpr bool LIN = D::LIN, DBL = D::DBL, SGL = D::SGL;
+    constexpr bool LIN = D::LIN, DBL = D::DBL, SGL = D::SGL, VEC = D::VEC;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int tid = threadIdx.x, NT = blockDim.x;
     const int J = a.J, G = a.G, np = a.np;
@@ -254,7 +257,7 @@ __global__ void __launch_bounds__(DIR_MAX_NT, 2) q2x_dir_kernel(const DirArgs a,
     int2* rec = reinterpret_cast<int2*>(smem_raw + (size_t)J * 48);
     longlong2* acc = reinterpret_cast<longlong2*>(smem_raw + (size_t)J * 48 + D::rec_bytes(a.p_max, T));
     __shared__ BatchTile s_tile;
-    __shared__ int s_more, s_ymax, s_r2, s_wmax, s_smax, s_bits[2][Q2X_P_MAX + 1];
+    __shared__ int s_more, s_ymax, s_r2, s_wmax, s_smax, s_bits[3][Q2X_P_MAX + 1];
     for (int i = tid; i < 6 * J; i += NT) dirs[i] = a.vec[i];
     const int g = tid / J, j = tid - g * J;
     const long long rnd = a.rnd;
@@ -269,7 +272,7 @@ __global__ void __launch_bounds__(DIR_MAX_NT, 2) q2x_dir_kernel(const DirArgs a,
             if (s_more) s_tile = a.tiles[ti];
             s_ymax = s_r2 = s_wmax = s_smax = 0;
         }
-        if (tid < 2 * (Q2X_P_MAX + 1)) (&s_bits[0][0])[tid] = 0;
+        if (tid < 3 * (Q2X_P_MAX + 1)) (&s_bits[0][0])[tid] = 0;
         __syncthreads();
         if (!s_more) break;
         const BatchTile t = s_tile;
@@ -321,6 +324,13 @@ __global__ void __launch_bounds__(DIR_MAX_NT, 2) q2x_dir_kernel(const DirArgs a,
 #pragma unroll
                 for (int k = 0; k < 3; ++k) {
                     s[k] = __ldg(a.kind.sigma + vid[k]);
+                    finite = finite && finite_bits(s[k]);
+                }
+            } else if (VEC) {
+                dens0 = 1.0;
+#pragma unroll
+                for (int k = 0; k < 3; ++k) {
+                    s[k] = __ldg(a.wvec + (int64_t)k * a.kind.n_elem + e);
                     finite = finite && finite_bits(s[k]);
                 }
             } else {
@@ -394,7 +404,7 @@ __global__ void __launch_bounds__(DIR_MAX_NT, 2) q2x_dir_kernel(const DirArgs a,
             }
             w = LIN ? J64 : J64 * dens0;
             wm = hi32(__double_as_longlong(w)) & 0x7fffffff;
-            if (LIN) {
+            if (LIN || VEC) {
 #pragma unroll
                 for (int k = 0; k < 3; ++k) sm = max(sm, hi32(__double_as_longlong(s[k])) & 0x7fffffff);
             }
@@ -403,11 +413,11 @@ __global__ void __launch_bounds__(DIR_MAX_NT, 2) q2x_dir_kernel(const DirArgs a,
         {
             const int m = __reduce_max_sync(0xffffffffu, r2i);
             const int mw = __reduce_max_sync(0xffffffffu, wm);
-            const int ms = LIN ? __reduce_max_sync(0xffffffffu, sm) : 0;
+            const int ms = (LIN || VEC) ? __reduce_max_sync(0xffffffffu, sm) : 0;
             if ((tid & 31) == 0) {
                 if (m) atomicMax(&s_r2, m);
                 if (mw) atomicMax(&s_wmax, mw);
-                if (LIN && ms) atomicMax(&s_smax, ms);
+                if ((LIN || VEC) && ms) atomicMax(&s_smax, ms);
             }
         }
         __syncthreads();
@@ -443,7 +453,7 @@ __global__ void __launch_bounds__(DIR_MAX_NT, 2) q2x_dir_kernel(const DirArgs a,
                     r[D::R_NRM + d] = make_int2(f.h, f.l);
                 }
             }
-            if (LIN) {
+            if (LIN || VEC) {
 #pragma unroll
                 for (int k = 0; k < 3; ++k) {  // half the scaled densities: below one also when rounded
                     const Fx f = fx_split(live ? dir_fixed((unsigned long long)__double_as_longlong(s[k]), es, 61) : 0);
@@ -487,7 +497,7 @@ __global__ void __launch_bounds__(DIR_MAX_NT, 2) q2x_dir_kernel(const DirArgs a,
                         }
                     }
                     Fx s1{}, s2{}, s3{};
-                    if (LIN) {
+                    if (LIN || VEC) {
                         s1 = as_fx(r[D::R_DENS]);
                         s2 = as_fx(r[D::R_DENS + 1]);
                         s3 = as_fx(r[D::R_DENS + 2]);
@@ -515,7 +525,17 @@ __global__ void __launch_bounds__(DIR_MAX_NT, 2) q2x_dir_kernel(const DirArgs a,
                         }
                         *p = o;
                     };
-                    if (SGL) put(at, Cx{W0, 0});
+                    // a vector density's three sums, the weights times the unit-density value
+                    auto put3 = [&](longlong2* p, const Cx& v, const CxH& vh, long long b) {
+                        const int st = (a.p_max + 1) * NT;
+                        put(p, Cx{mul1(s1, (int)v.re, vh.rh, -b, rnd), mul1(s1, (int)v.im, vh.ih, -b, rnd)});
+                        put(p + st, Cx{mul1(s2, (int)v.re, vh.rh, -b, rnd), mul1(s2, (int)v.im, vh.ih, -b, rnd)});
+                        put(p + 2 * st, Cx{mul1(s3, (int)v.re, vh.rh, -b, rnd), mul1(s3, (int)v.im, vh.ih, -b, rnd)});
+                    };
+                    if (VEC)
+                        put3(at, Cx{seed, 0}, CxH{high_of<0>(seed), 0}, dir_bias(1));
+                    else if (SGL)
+                        put(at, Cx{W0, 0});
                     if (DBL) put(at1, Cx{0, 0});
                     static_for<0, NL>([&](auto k_c) {
                         constexpr int k = decltype(k_c)::value, B = D::bias(k);
@@ -560,7 +580,10 @@ __global__ void __launch_bounds__(DIR_MAX_NT, 2) q2x_dir_kernel(const DirArgs a,
                             }
                             if (SGL) {
                                 at += NT;
-                                put(at, x[NL - 1]);
+                                if (VEC)
+                                    put3(at, x[NL - 1], h[NL - 1], 0);
+                                else
+                                    put(at, x[NL - 1]);
                             }
                         }
                     };
@@ -598,8 +621,8 @@ __global__ void __launch_bounds__(DIR_MAX_NT, 2) q2x_dir_kernel(const DirArgs a,
                 H += hi32(v);
                 Lo += (unsigned)(int)v;
             }
-            const bool second = !SGL || ly == 1;
-            if (n) H -= (long long)n_el * (second ? 1 : D::bias(NL - 1));
+            const bool once = VEC || !SGL || ly == 1;  // a product of the level's value: one bias
+            if (n) H -= (long long)n_el * (once ? 1 : D::bias(NL - 1));
             H += Lo >> 32;
             sums[i] = make_longlong2(H, Lo & 0xffffffffll);
             const int b = 64 - __clzll(H < 0 ? ~H : H);
@@ -627,7 +650,7 @@ __global__ void __launch_bounds__(DIR_MAX_NT, 2) q2x_dir_kernel(const DirArgs a,
         const bool direct = (t.flags & 1) != 0;
         for (int i = tid; i < np * D::LAYERS; i += NT) {
             const int ly = i / np, k = i - ly * np;
-            const bool second = !SGL || ly == 1;  // double layer
+            const bool second = !VEC && (!SGL || ly == 1);  // double layer
             const int desc = col_desc(k), n = desc & 31;
             double v = 0.0;
             if (n <= pL) {
@@ -652,7 +675,7 @@ __global__ void __launch_bounds__(DIR_MAX_NT, 2) q2x_dir_kernel(const DirArgs a,
                 int e2 = s_bits[ly][n] - 24 - 2 - a.seed_bits + DIR_EVENT * ((n >= a.event[0]) + (n >= a.event[1]) + (n >= a.event[2]) + (n >= a.event[3])) + (ew - 1022) +
                          (ns > 0 ? ns * (ex - 1022) : 0) + (KIND + 1) * Ej;
                 if (second) e2 += 1;
-                if (LIN) e2 += es - 1022 + 1;
+                if (LIN || VEC) e2 += es - 1022 + 1;
                 if (e2 > 1000 || e2 < -1000) {
                     const int h = max(-2000, min(2000, e2)) / 2;
                     v *= pow2d(h);
@@ -662,6 +685,7 @@ __global__ void __launch_bounds__(DIR_MAX_NT, 2) q2x_dir_kernel(const DirArgs a,
                 if ((desc >> (5 + a.norm)) & 1) v = -v;
                 if (wmax >= 0x7ff00000) v = __longlong_as_double(0x7ff8000000000000ll);
             }
+            if (VEC && a.coef[ly] == nullptr) continue;
             double* out = (direct ? a.coef[ly] + L * np : a.partial[ly] + t.slot * np) + k;
             *out = (direct && a.accumulate) ? *out + v : v;
         }
@@ -673,17 +697,18 @@ struct DirFns {
     cudaError_t (*occupancy)(int* blocks_per_sm, int p, int T);
 };
 // combos: 0 segments, 1-3 triangles constant density (single, double, both),
-// 4-6 linear density, 7 tetrahedra (the element kernel's order)
+// 4-6 linear density, 7 tetrahedra, 8 segments carrying a vector density (the
+// element kernel's order)
 const DirFns* dir_fns();
 // Threads of a CTA, and the elements a tile may hold: eight a group (the
 // number format's head room), at most one a thread (the frames).
-int dir_threads(int p);
-inline int dir_tile_elems(int p)
+int dir_threads(int p, bool vec);
+inline int dir_tile_elems(int p, bool vec)
 {
-    const int nt = dir_threads(p), t = 8 * (nt / (p + 1));
+    const int nt = dir_threads(p, vec), t = 8 * (nt / (p + 1));
     return t < nt ? t : nt;
 }
 // Fills the tables, group counts and number format of a call (a.p_max set).
-cudaError_t dir_setup(DirArgs& a, int kind, int dens);
+cudaError_t dir_setup(DirArgs& a, int kind, int dens, bool vec);
 
 }  // namespace q2x

@@ -124,3 +124,43 @@ def test_accumulate_and_repeat(q2x):
     acc = base.clone()
     plan.triangles(*args, coef_single=acc, accumulate=True)
     assert torch.equal(acc, base + one)
+
+
+@pytest.mark.parametrize("p", [0, 1, 6, 12, 16, 20])
+def test_vector_density(q2x, p):
+    """The three components of a line current, at tile edges of the 128-thread
+    CTAs, with a component that vanishes and one far smaller than the others."""
+    import torch
+    full = min(8 * (128 // (p + 1)), 128)
+    prob = random_problem("segment", [1, full - 1, 0, full, full + 1, 2 * full + 3, 5], seed=p + 9, p=p)
+    rng = np.random.default_rng(p)
+    cur = rng.uniform(-1, 1, size=(3, prob["idx"].shape[1]))
+    cur[1, :60] = 0.0
+    cur[2] *= 1e-6
+    d = {k: torch.from_numpy(np.ascontiguousarray(v)).cuda() for k, v in dict(prob, cur=cur).items() if hasattr(v, "dtype")}
+    plan = q2x.Plan(p)
+    got = plan.segments_vector(d["vxyz"], d["idx"], d["cur"], d["leaf_off"], d["leaf_c"], d["leaf_rho"], d["leaf_p"])
+    base = torch.rand_like(got)
+    acc = base.clone()
+    plan.segments_vector(d["vxyz"], d["idx"], d["cur"], d["leaf_off"], d["leaf_c"], d["leaf_rho"], d["leaf_p"],
+                         coef3=acc, accumulate=True)
+    assert torch.equal(acc, base + got)
+    one = torch.ones_like(d["sigma"])
+    leaf_of = np.repeat(np.arange(len(prob["leaf_off"]) - 1), np.diff(prob["leaf_off"]))
+    t = lambda x: torch.from_numpy(np.ascontiguousarray(x)).cuda()
+    rows = plan.segments(d["vxyz"], d["idx"], one, None, t(prob["leaf_c"][:, leaf_of]), t(prob["leaf_rho"][leaf_of]))
+    ref = plan.leaf_reduce_weighted(rows, p, d["leaf_off"], d["cur"]).cpu().numpy()
+    plan.sync()
+    # the components share one scale, the largest current of the leaf: errors
+    # against the largest coefficient of the degree over the three components
+    top = _degree_max(np.abs(ref).max(axis=0), p)
+    for k in range(3):
+        assert np.all(np.abs(got[k].cpu().numpy() - ref[k]) <= 1e-12 * np.maximum(top, 1e-300)), k
+
+
+def _degree_max(a, p):
+    """Per leaf and column, the largest magnitude over the column's degree."""
+    out = np.zeros_like(a)
+    for n in range(p + 1):
+        out[:, n * n:(n + 1) ** 2] = a[:, n * n:(n + 1) ** 2].max(axis=1, keepdims=True)
+    return out
