@@ -303,8 +303,8 @@ void leaf_tile_carve(unsigned char* p, int64_t n_elem, int64_t n_leaves, int np,
 }
 
 // FP64 leaf sums of one element set by the direction kernels
-q2x_status run_directions(q2x_plan_t plan, q2x::DirArgs& a, int kind, int dens, int combo, int T, int64_t n_elem,
-                          int64_t n_vert, const double* vxyz, const int32_t* idx, const double* sigma,
+q2x_status run_directions(q2x_plan_t plan, q2x::DirArgs& a, int combo, const q2x::DirShape& shape,
+                          int64_t n_elem,                          int64_t n_vert, const double* vxyz, const int32_t* idx, const double* sigma,
                           int64_t n_leaves, const int64_t* leaf_off, const double* leaf_c, const int32_t* leaf_p,
                           double* coef0, double* coef1, int accumulate, const double* wvec, double* coef2)
 {
@@ -317,10 +317,10 @@ q2x_status run_directions(q2x_plan_t plan, q2x::DirArgs& a, int kind, int dens, 
     const int layers = wvec ? 3 : out[1] ? 2 : 1;
     q2x::LeafTileWork w;
     double* partial[3] = {nullptr, nullptr, nullptr};
-    leaf_tile_carve(static_cast<unsigned char*>(plan->ws), n_elem, n_leaves, np, T, layers, w, partial);
+    leaf_tile_carve(static_cast<unsigned char*>(plan->ws), n_elem, n_leaves, np, shape.T, layers, w, partial);
     const int64_t nb = (n_leaves + 1 + 255) / 256;
     check_leaf_off_kernel<<<(unsigned)nb, 256, 0, plan->stream>>>(leaf_off, n_leaves, n_elem, plan->d_err);
-    cudaError_t e = q2x::leaf_tiles_build(leaf_off, n_leaves, T, 0, 0, w, plan->stream);
+    cudaError_t e = q2x::leaf_tiles_build(leaf_off, n_leaves, shape.T, 0, 0, w, plan->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(w.counter, 0, sizeof(unsigned long long), plan->stream);
     if (e != cudaSuccess) return cuda_fail(plan, e, "leaf tile list");
     a.kind = q2x::BatchKind{n_elem, n_vert, vxyz, vxyz + n_vert, vxyz + 2 * n_vert, idx, sigma};
@@ -339,10 +339,10 @@ q2x_status run_directions(q2x_plan_t plan, q2x::DirArgs& a, int kind, int dens, 
         a.partial[l] = partial[l];
         a.coef[l] = out[l];
     }
-    const q2x::DirFns& f = q2x::dir_fns()[combo];
-    int& occ = plan->dir_occ[combo];
+    const q2x::DirFns& f = q2x::dir_fns(shape.cls, combo);
+    int& occ = plan->dir_occ[shape.nt / 32][combo];
     if (occ == 0) {
-        e = f.occupancy(&occ, plan->p_max, T);
+        e = f.occupancy(&occ, plan->p_max, shape.nt, shape.T);
         if (e != cudaSuccess) return cuda_fail(plan, e, "direction kernel occupancy query");
         if (occ <= 0) return fail(plan, Q2X_ERR_CUDA, "direction kernel does not fit on the device");
     }
@@ -354,7 +354,7 @@ q2x_status run_directions(q2x_plan_t plan, q2x::DirArgs& a, int kind, int dens, 
         cudaEventRecord(ev0, plan->stream);
     }
     const int64_t grid = std::min<int64_t>((int64_t)occ * plan->num_sms, w.max_tiles);
-    e = f.launch(a, T, (int)grid, plan->stream);
+    e = f.launch(a, shape.nt, shape.T, (int)grid, plan->stream);
     if (e != cudaSuccess) return cuda_fail(plan, e, "direction kernel launch");
     if (plan->timing) {
         cudaEventRecord(ev1, plan->stream);
@@ -442,20 +442,19 @@ q2x_status run_elements(q2x_plan_t plan, int kind, int dens, int64_t n_elem, int
     // (q2x_dir.cuh), within the same workspace bound
     const bool dirs = prec == 0 && leaf_off && n_leaves < ((int64_t)1 << 31);
     q2x::DirArgs da{};
-    int dir_T = 0;
     const int dir_layers = vec ? 3 : (coef0 ? 1 : 0) + (dbl ? 1 : 0);
+    const q2x::DirShape shape = q2x::dir_shape(plan->p_max, dir_layers, n_elem, n_leaves);
     size_t dir_bytes = 0;
     if (dirs) {
         da.p_max = plan->p_max;
-        e = q2x::dir_setup(da, kind, dens, vec);
-        dir_T = q2x::dir_tile_elems(plan->p_max, vec);
+        e = q2x::dir_setup(da, kind, dens, shape.nt);
         if (e != cudaSuccess) return cuda_fail(plan, e, "direction tables");
-        dir_bytes = leaf_tile_ws_bytes(n_elem, n_leaves, np, dir_T, dir_layers);
+        dir_bytes = leaf_tile_ws_bytes(n_elem, n_leaves, np, shape.T, dir_layers);
     }
     if (dirs && dir_bytes <= ((size_t)8 << 30)) {
         q2x_status st = ensure_ws(plan, dir_bytes);
         if (st != Q2X_OK) return st;
-        return run_directions(plan, da, kind, dens, combo, dir_T, n_elem, n_vert, vxyz, idx, sigma, n_leaves, leaf_off,
+        return run_directions(plan, da, combo, shape, n_elem, n_vert, vxyz, idx, sigma, n_leaves, leaf_off,
                               leaf_c, leaf_p, coef0, dbl || vec ? coef1 : nullptr, accumulate, wvec, coef2);
     }
     const int64_t resident_warps = (int64_t)occ * wpc * plan->num_sms;
@@ -747,11 +746,13 @@ q2x_status q2x_reserve(q2x_plan_t plan, int64_t n_elem, int64_t n_leaves)
     // worst case: one range per 32 elements; FP64 partials in both precisions
     const int64_t n_ranges = (n_elem + 31) / 32;
     const size_t elem = align_up(sizeof(double) * (size_t)n_ranges * 2 * 3 * np, 256);
-    size_t tile = plan->prec == 1 ? leaf_tile_ws_bytes(n_elem, n_leaves, np, kLeafTileElems)
-                                  : std::max(leaf_tile_ws_bytes(n_elem, n_leaves, np,
-                                                                q2x::dir_tile_elems(plan->p_max, false), 2),
-                                             leaf_tile_ws_bytes(n_elem, n_leaves, np,
-                                                                q2x::dir_tile_elems(plan->p_max, true), 3));
+    size_t tile = 0;
+    if (plan->prec == 1)
+        tile = leaf_tile_ws_bytes(n_elem, n_leaves, np, kLeafTileElems);
+    else
+        for (int layers = 1; layers <= 3; ++layers)
+            tile = std::max(tile, leaf_tile_ws_bytes(n_elem, n_leaves, np,
+                                                     q2x::dir_shape(plan->p_max, layers, n_elem, n_leaves).T, layers));
     if (tile > ((size_t)8 << 30)) tile = 0;  // such calls run the element kernel
     const size_t bytes = std::max(elem, tile) + align_up(sizeof(double) * (size_t)n_leaves, 256) +
                          align_up(sizeof(int) * (size_t)n_leaves, 256);

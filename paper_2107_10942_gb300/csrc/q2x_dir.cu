@@ -10,56 +10,76 @@ namespace q2x {
 
 namespace {
 
-template <int KIND, int DENS, int OUTS>
-cudaError_t dir_attr(int p, int T, size_t* smem)
+template <int KIND, int DENS, int OUTS, int MAX_NT>
+cudaError_t dir_attr(int p, int nt, int T, size_t* smem)
 {
-    *smem = DirCfg<KIND, DENS, OUTS>::smem(p, T, dir_threads(p, (OUTS & 4) != 0));
-    return cudaFuncSetAttribute(q2x_dir_kernel<KIND, DENS, OUTS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    *smem = DirCfg<KIND, DENS, OUTS>::smem(p, T, nt);
+    return cudaFuncSetAttribute(q2x_dir_kernel<KIND, DENS, OUTS, MAX_NT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 (int)*smem);
 }
 
-template <int KIND, int DENS, int OUTS>
-cudaError_t dir_launch(const DirArgs& a, int T, int grid, cudaStream_t st)
+template <int KIND, int DENS, int OUTS, int MAX_NT>
+cudaError_t dir_launch(const DirArgs& a, int nt, int T, int grid, cudaStream_t st)
 {
     size_t smem;
-    cudaError_t e = dir_attr<KIND, DENS, OUTS>(a.p_max, T, &smem);
+    cudaError_t e = dir_attr<KIND, DENS, OUTS, MAX_NT>(a.p_max, nt, T, &smem);
     if (e != cudaSuccess) return e;
-    q2x_dir_kernel<KIND, DENS, OUTS><<<grid, dir_threads(a.p_max, (OUTS & 4) != 0), smem, st>>>(a, T);
+    q2x_dir_kernel<KIND, DENS, OUTS, MAX_NT><<<grid, nt, smem, st>>>(a, T);
     return cudaGetLastError();
 }
 
-template <int KIND, int DENS, int OUTS>
-cudaError_t dir_occupancy(int* blocks, int p, int T)
+template <int KIND, int DENS, int OUTS, int MAX_NT>
+cudaError_t dir_occupancy(int* blocks, int p, int nt, int T)
 {
     size_t smem;
-    cudaError_t e = dir_attr<KIND, DENS, OUTS>(p, T, &smem);
+    cudaError_t e = dir_attr<KIND, DENS, OUTS, MAX_NT>(p, nt, T, &smem);
     if (e != cudaSuccess) return e;
-    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks, q2x_dir_kernel<KIND, DENS, OUTS>,
-                                                         dir_threads(p, (OUTS & 4) != 0), smem);
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks, q2x_dir_kernel<KIND, DENS, OUTS, MAX_NT>, nt, smem);
 }
 
-#define Q2X_DIR_FNS(K, D, O) {&dir_launch<K, D, O>, &dir_occupancy<K, D, O>}
+#define Q2X_DIR_FNS(K, D, O, M) {&dir_launch<K, D, O, M>, &dir_occupancy<K, D, O, M>}
+#define Q2X_DIR_ROW(M)                                                                                       \
+    {Q2X_DIR_FNS(KIND_SEG, DENS_CONST, 1, M),  Q2X_DIR_FNS(KIND_TRI, DENS_CONST, 1, M),                      \
+     Q2X_DIR_FNS(KIND_TRI, DENS_CONST, 2, M),  Q2X_DIR_FNS(KIND_TRI, DENS_CONST, 3, M),                      \
+     Q2X_DIR_FNS(KIND_TRI, DENS_LINEAR, 1, M), Q2X_DIR_FNS(KIND_TRI, DENS_LINEAR, 2, M),                     \
+     Q2X_DIR_FNS(KIND_TRI, DENS_LINEAR, 3, M), Q2X_DIR_FNS(KIND_TET, DENS_CONST, 1, M),                      \
+     Q2X_DIR_FNS(KIND_SEG, DENS_CONST, 4, M)}
 
 }  // namespace
 
-// 256 threads, 17 directions: 255 at work at p = 16.  Smaller CTAs overlap
-// their phases better but map twice as many tiles to coefficients (level-9
-// sphere, p = 16: 11.4 ms with 256 threads, 11.6 with 128, 12.6 with 160).
-// The three sums of a vector density take three times the shared memory: 128.
-int dir_threads(int, bool vec) { return vec ? 128 : 256; }
-
-const DirFns* dir_fns()
+const DirFns& dir_fns(int cls, int combo)
 {
-    static const DirFns f[9] = {
-        Q2X_DIR_FNS(KIND_SEG, DENS_CONST, 1),  Q2X_DIR_FNS(KIND_TRI, DENS_CONST, 1),
-        Q2X_DIR_FNS(KIND_TRI, DENS_CONST, 2),  Q2X_DIR_FNS(KIND_TRI, DENS_CONST, 3),
-        Q2X_DIR_FNS(KIND_TRI, DENS_LINEAR, 1), Q2X_DIR_FNS(KIND_TRI, DENS_LINEAR, 2),
-        Q2X_DIR_FNS(KIND_TRI, DENS_LINEAR, 3), Q2X_DIR_FNS(KIND_TET, DENS_CONST, 1),
-        Q2X_DIR_FNS(KIND_SEG, DENS_CONST, 4)};
-    return f;
+    static const DirFns f[2][9] = {Q2X_DIR_ROW(256), Q2X_DIR_ROW(128)};
+    return f[cls][combo];
 }
 
-cudaError_t dir_setup(DirArgs& a, int kind, int dens, bool vector)
+// 256 threads where two such CTAs fit an SM's shared memory (p = 16, single
+// layer: 255 of them at work), else the most that do (constant density, both
+// layers, p = 12: 1.76 ms with 192 threads, 2.11 with one CTA of 256); a vector
+// density takes one CTA of 256 as long as that fits (2M segments, p = 12: 4.3
+// ms, 4.7 with two of 160).  Where leaves are small a tile keeps few groups
+// busy and its frames bound it, so more and smaller CTAs overlap better
+// (800,000 triangles, p = 16: 13 a leaf 2.5 ms with 128 threads, 3.3 with 256;
+// 3 a leaf 5.7 with 64, 8.9 with 256; p = 8: 13 a leaf 0.80 with 64, 1.55 with
+// 256; 53 a leaf 256 is ahead at p = 12, 1.12 against 1.18 ms, and 40 tetrahedra a
+// leaf at p = 10, 0.26 against 0.31, but behind at p = 8, 0.70 against 0.56).
+DirShape dir_shape(int p, int layers, int64_t n_elem, int64_t n_leaves)
+{
+    const double mean = (double)n_elem / (double)std::max<int64_t>(n_leaves, 1);
+    DirShape s{0, 256, 0};
+    // accumulators, directions and about 8 groups' records of 128 bytes
+    auto smem = [&](int nt) { return (size_t)(p + 1) * (16 * layers * nt + 48) + (size_t)nt / (p + 1) * 1024; };
+    const size_t most = layers == 3 ? 200 * 1024 : 110 * 1024;
+    while (s.nt > 128 && smem(s.nt) > most) s.nt -= 32;
+    if (mean < (p >= 10 ? 32.0 : 96.0) && layers < 3) {
+        s.nt = mean < (p >= 10 ? 5.0 : 20.0) ? 64 : 128;
+        s.cls = (p >= 12 && s.nt == 128) ? 0 : 1;
+    }
+    s.T = dir_tile_elems(p, s.nt);
+    return s;
+}
+
+cudaError_t dir_setup(DirArgs& a, int kind, int dens, int nt)
 {
     const int p = a.p_max;
     void *vec, *inv, *eighth, *pw, *col;
@@ -75,7 +95,7 @@ cudaError_t dir_setup(DirArgs& a, int kind, int dens, bool vector)
     a.pw = static_cast<const double*>(pw);
     a.col = static_cast<const double*>(col);
     a.J = p + 1;
-    a.G = dir_threads(p, vector) / a.J;
+    a.G = nt / a.J;
     a.rnd = (long long)((1ull << 63) + (1ull << 31));
     // Bound of a level's value over the seed's (|u| < 1): the dimension's
     // binomial, for linear density (n+1)(n+2)(n+3)/2 of a half.  Seeds start at

@@ -27,9 +27,9 @@
 //
 // What bounds it: the integer multiplies, 36 per step of the triangle chain
 // (190 cycles with the additions between them; 196 measured in a loop of its
-// own), then the tile's other phases: of the level-9 sphere's 11.4 ms at p =
-// 16 the recurrences are 62 %, the map to coefficients 16 %, the frames 12 %,
-// the sums over groups 8 %.  The FP64 row kernel took 36.2 ms.
+// own), then the tile's other phases: of the level-9 sphere's 11.2 ms at p =
+// 16 the recurrences are 64 %, the map to coefficients and the frames 13 %
+// each, the sums over groups 8 %.  The FP64 row kernel took 36.2 ms.
 //
 // One CTA per tile of one leaf's elements: thread t < G J owns direction
 // t mod J and elements t / J, t / J + G, .. (at most eight, the number
@@ -212,7 +212,6 @@ struct DirArgs {
 
 // What one CTA's shared memory holds: the directions, the elements' records
 // (later the sums), the accumulators [layer][degree][thread] of 16 bytes.
-constexpr int DIR_MAX_NT = 256;
 constexpr int DIR_EVENT = 3;  // bits dropped when the values' bound has grown by them
 template <int KIND, int DENS, int OUTS>
 struct DirCfg {
@@ -231,8 +230,8 @@ struct DirCfg {
     static constexpr int REC = R_SEED + 1;
     __host__ __device__ static constexpr size_t rec_bytes(int p, int T)
     {
-        // the records' space is reused for the sums: 12 bytes each, then 8
-        const size_t a = (size_t)T * REC * 8, s = (size_t)(p + 1) * 2 * (p + 1) * LAYERS * 16;
+        // the records' space is reused for the sums
+        const size_t a = (size_t)T * REC * 8, s = (size_t)(p + 1) * 2 * (p + 1) * LAYERS * 8;
         return ((a > s ? a : s) + 15) / 16 * 16;
     }
     __host__ __device__ static constexpr size_t smem(int p, int T, int nt)
@@ -243,8 +242,9 @@ struct DirCfg {
 
 __device__ __forceinline__ Fx as_fx(int2 v) { return Fx{v.x, v.y}; }
 
-template <int KIND, int DENS, int OUTS>
-__global__ void __launch_bounds__(DIR_MAX_NT, 2) q2x_dir_kernel(const DirArgs a, int T)
+// MAX_NT 256: two CTAs of up to 128 registers a thread; 128: six of up to 80.
+template <int KIND, int DENS, int OUTS, int MAX_NT>
+__global__ void __launch_bounds__(MAX_NT, MAX_NT == 256 ? 2 : 6) q2x_dir_kernel(const DirArgs a, int T)
 {
     using D = DirCfg<KIND, DENS, OUTS>;
     constexpr int NV = D::NV;
@@ -272,7 +272,6 @@ __global__ void __launch_bounds__(DIR_MAX_NT, 2) q2x_dir_kernel(const DirArgs a,
             if (s_more) s_tile = a.tiles[ti];
             s_ymax = s_r2 = s_wmax = s_smax = 0;
         }
-        if (tid < 3 * (Q2X_P_MAX + 1)) (&s_bits[0][0])[tid] = 0;
         __syncthreads();
         if (!s_more) break;
         const BatchTile t = s_tile;
@@ -607,60 +606,71 @@ __global__ void __launch_bounds__(DIR_MAX_NT, 2) q2x_dir_kernel(const DirArgs a,
         }
         __syncthreads();
 
-        // ---- sums over the groups: 96-bit, then 56 bits of each degree's largest
-        const int n_val = pL >= 0 ? (pL + 1) * 2 * J : 0;  // per layer
+        // ---- sums over the groups, 96-bit, cut to 56 bits of each degree's
+        // largest: a warp per degree and layer, so that the largest is a warp
+        // reduction
         const int Ga = min(G, n_el);
-        longlong2* sums = reinterpret_cast<longlong2*>(rec);  // (high 64, low 32)
-        for (int i = tid; i < n_val * D::LAYERS; i += NT) {
-            const int ly = i / n_val, r = i - ly * n_val;
-            const int n = r / (2 * J), q = r - n * 2 * J;
-            const long long* p = reinterpret_cast<const long long*>(acc + (ly * (a.p_max + 1) + n) * NT) + q;
-            long long H = 0, Lo = 0;
-            for (int k = 0; k < Ga; ++k) {
-                const long long v = p[(size_t)k * 2 * J];
-                H += hi32(v);
-                Lo += (unsigned)(int)v;
-            }
+        int2* sums = rec;  // [layer][degree][2 J]
+        for (int r = tid >> 5; r < (pL + 1) * D::LAYERS; r += NT >> 5) {
+            int ly = 0, n = r;
+            while (n > pL) n -= pL + 1, ++ly;
             const bool once = VEC || !SGL || ly == 1;  // a product of the level's value: one bias
-            if (n) H -= (long long)n_el * (once ? 1 : D::bias(NL - 1));
-            H += Lo >> 32;
-            sums[i] = make_longlong2(H, Lo & 0xffffffffll);
-            const int b = 64 - __clzll(H < 0 ? ~H : H);
-            if (b) atomicMax(&s_bits[ly][n], b);
-        }
-        __syncthreads();
-        for (int i = tid; i < n_val * D::LAYERS; i += NT) {
-            const int ly = i / n_val, r = i - ly * n_val;
-            const int n = r / (2 * J);
-            const longlong2 v = sums[i];
-            const int sh = s_bits[ly][n] - 24;  // |value| < 2^(bits + 32) -> below 2^56
-            long long o;
-            if (sh <= 0)
-                o = (long long)(((unsigned long long)v.x << 32) | (unsigned long long)v.y) << -sh;
-            else if (sh < 32)
-                o = (long long)(((unsigned long long)v.x << (32 - sh)) | ((unsigned long long)v.y >> sh));
-            else
-                o = v.x >> (sh - 32);
-            const int hq = (int)((o + (1ll << 27)) >> 28);
-            reinterpret_cast<int2*>(sums + i)[0] = make_int2(hq, (int)(o - ((long long)hq << 28)));
+            const int bias = n ? n_el * (once ? 1 : D::bias(NL - 1)) : 0;
+            long long H[2] = {0, 0}, Lo[2] = {0, 0};
+            int bits = 0;
+#pragma unroll
+            for (int c = 0; c < 2; ++c) {  // 2 J <= 42 columns
+                const int q = (tid & 31) + 32 * c;
+                if (q < 2 * J) {
+                    const long long* p = reinterpret_cast<const long long*>(acc + (ly * (a.p_max + 1) + n) * NT) + q;
+#pragma unroll 4
+                    for (int k = 0; k < Ga; ++k) {
+                        const long long v = p[k * 2 * J];
+                        H[c] += hi32(v);
+                        Lo[c] += (unsigned)(int)v;
+                    }
+                    H[c] += (Lo[c] >> 32) - bias;
+                    bits = max(bits, 64 - __clzll(H[c] < 0 ? ~H[c] : H[c]));
+                }
+            }
+            bits = __reduce_max_sync(0xffffffffu, bits);  // |value| < 2^(bits + 32) -> below 2^56
+            const int sh = bits - 24;
+#pragma unroll
+            for (int c = 0; c < 2; ++c) {
+                const int q = (tid & 31) + 32 * c;
+                if (q < 2 * J) {
+                    const unsigned long long hi = (unsigned long long)H[c], lo = (unsigned)(int)Lo[c];
+                    long long o;
+                    if (sh <= 0)
+                        o = (long long)((hi << 32) | lo) << -sh;
+                    else if (sh < 32)
+                        o = (long long)((hi << (32 - sh)) | (lo >> sh));
+                    else
+                        o = H[c] >> (sh - 32);
+                    const int hq = (int)((o + (1ll << 27)) >> 28);
+                    sums[r * 2 * J + q] = make_int2(hq, (int)(o - ((long long)hq << 28)));
+                }
+            }
+            if ((tid & 31) == 0) s_bits[ly][n] = bits;
         }
         __syncthreads();
 
         // ---- coefficients: the left inverse's row of each packed column
         const bool direct = (t.flags & 1) != 0;
         for (int i = tid; i < np * D::LAYERS; i += NT) {
-            const int ly = i / np, k = i - ly * np;
+            int ly = 0, k = i;
+            while (k >= np) k -= np, ++ly;
             const bool second = !VEC && (!SGL || ly == 1);  // double layer
             const int desc = col_desc(k), n = desc & 31;
             double v = 0.0;
             if (n <= pL) {
                 const int2* P = a.inv + k;
-                const longlong2* S = sums + ly * n_val + n * 2 * J;
+                const int2* S = sums + (ly * (pL + 1) + n) * 2 * J;
                 long long hh = 0, mid = 1ll << 27;
-#pragma unroll 4
+#pragma unroll 8
                 for (int q = 0; q < 2 * J; ++q) {
-                    const int2 c = __ldg(P + (size_t)q * np);
-                    const int2 x = *reinterpret_cast<const int2*>(S + q);
+                    const int2 c = __ldg(P + q * np);
+                    const int2 x = S[q];
                     mid = madw(c.x, x.y, mid);
                     mid = madw(c.y, x.x, mid);
                     hh = madw(c.x, x.x, hh);
@@ -693,22 +703,26 @@ __global__ void __launch_bounds__(DIR_MAX_NT, 2) q2x_dir_kernel(const DirArgs a,
 }
 
 struct DirFns {
-    cudaError_t (*launch)(const DirArgs&, int T, int grid, cudaStream_t);
-    cudaError_t (*occupancy)(int* blocks_per_sm, int p, int T);
+    cudaError_t (*launch)(const DirArgs&, int nt, int T, int grid, cudaStream_t);
+    cudaError_t (*occupancy)(int* blocks_per_sm, int p, int nt, int T);
 };
-// combos: 0 segments, 1-3 triangles constant density (single, double, both),
-// 4-6 linear density, 7 tetrahedra, 8 segments carrying a vector density (the
-// element kernel's order)
-const DirFns* dir_fns();
-// Threads of a CTA, and the elements a tile may hold: eight a group (the
-// number format's head room), at most one a thread (the frames).
-int dir_threads(int p, bool vec);
-inline int dir_tile_elems(int p, bool vec)
+// [CTA class: 0 up to 256 threads, 1 up to 128][combo]; combos: 0 segments, 1-3
+// triangles constant density (single, double, both), 4-6 linear density, 7
+// tetrahedra, 8 segments carrying a vector density (the element kernel's order)
+const DirFns& dir_fns(int cls, int combo);
+// A call's CTAs: class, threads, elements per tile.
+struct DirShape {
+    int cls, nt, T;
+};
+DirShape dir_shape(int p, int layers, int64_t n_elem, int64_t n_leaves);
+// Elements a tile may hold: eight a group (the number format's head room), at
+// most one a thread (the frames).
+inline int dir_tile_elems(int p, int nt)
 {
-    const int nt = dir_threads(p, vec), t = 8 * (nt / (p + 1));
+    const int t = 8 * (nt / (p + 1));
     return t < nt ? t : nt;
 }
 // Fills the tables, group counts and number format of a call (a.p_max set).
-cudaError_t dir_setup(DirArgs& a, int kind, int dens, bool vec);
+cudaError_t dir_setup(DirArgs& a, int kind, int dens, int nt);
 
 }  // namespace q2x

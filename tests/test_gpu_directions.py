@@ -55,13 +55,23 @@ def check(prob, p, got, ref):
             assert norm_err(g.cpu().numpy(), r.cpu().numpy(), p, prob["leaf_rho"], layer) <= 1e-12
 
 
+def edge_sizes(p, small):
+    """Leaf sizes about the edges of a group, a full tile and two tiles for the
+    CTA sizes of small leaves (64, 128 threads; many tiny leaves among them) or
+    of large ones (128 to 256)."""
+    sizes = [1, 0, 2, 7, 8, 9, 33]
+    for nt in (64, 128) if small else (128, 160, 192, 256):
+        groups = max(1, nt // (p + 1))
+        full = min(8 * groups, nt)
+        sizes += [max(groups - 1, 1), groups, groups + 1, full - 1, full, full + 1, 0, min(2 * full + 1, 600)]
+    return sizes + ([1, 2, 3, 1, 0, 5] * 40 if small else [500, 700])
+
+
 @pytest.mark.parametrize("kind,density", KINDS)
+@pytest.mark.parametrize("small", [True, False])
 @pytest.mark.parametrize("p", [0, 1, 2, 5, 11, 13, 15, 18, 20])
-def test_tile_edges(q2x, kind, density, p):
-    groups = 256 // (p + 1)
-    full = min(8 * groups, 256)
-    sizes = [1, groups - 1, groups, groups + 1, full - 1, full, 0, full + 1, min(2 * full + 1, 600), 2, 7, 8, 9, 33]
-    prob = random_problem(kind, sizes, seed=p + 50, p=p, density=density)
+def test_tile_edges(q2x, kind, density, p, small):
+    prob = random_problem(kind, edge_sizes(p, small), seed=p + 50, p=p, density=density)
     layers = (True, kind == "triangle")
     check(prob, p, *both(q2x, prob, p, layers))
 
@@ -128,11 +138,9 @@ def test_accumulate_and_repeat(q2x):
 
 @pytest.mark.parametrize("p", [0, 1, 6, 12, 16, 20])
 def test_vector_density(q2x, p):
-    """The three components of a line current, at tile edges of the 128-thread
-    CTAs, with a component that vanishes and one far smaller than the others."""
+    """The three components of a line current, at tile edges, with a component that vanishes and one far smaller than the others."""
     import torch
-    full = min(8 * (128 // (p + 1)), 128)
-    prob = random_problem("segment", [1, full - 1, 0, full, full + 1, 2 * full + 3, 5], seed=p + 9, p=p)
+    prob = random_problem("segment", edge_sizes(p, False), seed=p + 9, p=p)
     rng = np.random.default_rng(p)
     cur = rng.uniform(-1, 1, size=(3, prob["idx"].shape[1]))
     cur[1, :60] = 0.0
