@@ -79,9 +79,8 @@ DirShape dir_shape(int p, int layers, int64_t n_elem, int64_t n_leaves)
     return s;
 }
 
-cudaError_t dir_setup(DirArgs& a, int kind, int dens, int nt)
+cudaError_t dir_tables(int p, DirTables* t)
 {
-    const int p = a.p_max;
     void *vec, *inv, *eighth, *pw, *col;
     cudaError_t e = cudaGetSymbolAddress(&vec, g_dir_vec);
     if (e == cudaSuccess) e = cudaGetSymbolAddress(&inv, g_dir_inv);
@@ -89,11 +88,25 @@ cudaError_t dir_setup(DirArgs& a, int kind, int dens, int nt)
     if (e == cudaSuccess) e = cudaGetSymbolAddress(&pw, g_dir_pow);
     if (e == cudaSuccess) e = cudaGetSymbolAddress(&col, g_dir_col);
     if (e != cudaSuccess) return e;
-    a.vec = static_cast<const int2*>(vec) + h_dir_vec_off[p];
-    a.inv = static_cast<const int2*>(inv) + h_dir_inv_off[p];
-    a.eighth = static_cast<const int2*>(eighth);
-    a.pw = static_cast<const double*>(pw);
-    a.col = static_cast<const double*>(col);
+    t->vec = static_cast<const int2*>(vec) + h_dir_vec_off[p];
+    t->inv = static_cast<const int2*>(inv) + h_dir_inv_off[p];
+    t->eighth = static_cast<const int2*>(eighth);
+    t->pw = static_cast<const double*>(pw);
+    t->col = static_cast<const double*>(col);
+    return cudaSuccess;
+}
+
+cudaError_t dir_setup(DirArgs& a, int kind, int dens, int nt)
+{
+    const int p = a.p_max;
+    DirTables t;
+    cudaError_t e = dir_tables(p, &t);
+    if (e != cudaSuccess) return e;
+    a.vec = t.vec;
+    a.inv = t.inv;
+    a.eighth = t.eighth;
+    a.pw = t.pw;
+    a.col = t.col;
     a.J = p + 1;
     a.G = nt / a.J;
     a.rnd = (long long)((1ull << 63) + (1ull << 31));

@@ -722,6 +722,13 @@ inline int dir_tile_elems(int p, int nt)
     const int t = 8 * (nt / (p + 1));
     return t < nt ? t : nt;
 }
+// The device tables of degree bound p: vectors [J][6], left inverse [2 J][np],
+// 2^(k/8 - 1) [15], 2^(-k n / 8) [15][24], column constants [norm][d][441].
+struct DirTables {
+    const int2 *vec, *inv, *eighth;
+    const double *pw, *col;
+};
+cudaError_t dir_tables(int p, DirTables* t);
 // Fills the tables, group counts and number format of a call (a.p_max set).
 cudaError_t dir_setup(DirArgs& a, int kind, int dens, int nt);
 
