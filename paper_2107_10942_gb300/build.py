@@ -44,12 +44,12 @@ def build(force: bool = False, jobs: int | None = None, verbose: bool = False) -
     srcs = sorted(f for f in os.listdir(CSRC) if f.endswith(".cu"))
     headers = [os.path.join(CSRC, f) for f in os.listdir(CSRC) if f.endswith((".cuh", ".h"))]
     headers.append(os.path.join(ROOT, "include", "q2x.h"))
-    gen = os.path.join(HERE, "gen_directions.py")
-    table = os.path.join(OUT, "q2x_dirs_table.inc")
-    if force or _stale(table, [gen]):
-        subprocess.run([sys.executable, gen, table + ".tmp"], check=True)
-        os.replace(table + ".tmp", table)
-    headers.append(table)
+    for name, out in (("gen_directions.py", "q2x_dirs_table.inc"), ("gen_nearfield.py", "q2x_nf_table.inc")):
+        gen, table = os.path.join(HERE, name), os.path.join(OUT, out)
+        if force or _stale(table, [gen]):
+            subprocess.run([sys.executable, gen, table + ".tmp"], check=True)
+            os.replace(table + ".tmp", table)
+        headers.append(table)
     objs = []
     todo = []
     for s in srcs:

@@ -29,6 +29,15 @@
 #include "q2x.h"
 #include "q2x_plan.h"
 
+#define Q2X_NF_TABLE static __device__ const
+#include "q2x_nf_table.inc"  // written by gen_nearfield.py
+namespace q2x {
+using ::NF_LN2_55;
+using ::NF_LN2_63;
+using ::NF_PI_61;
+}  // namespace q2x
+#include "q2x_nfmath.cuh"
+
 namespace q2x {
 
 constexpr double NF_INV_4PI = 0.079577471545947667884;
@@ -68,32 +77,34 @@ __device__ __forceinline__ V3 scale(V3 a, double s) { return V3{a.x * s, a.y * s
 // With N/D the ratio, N - D = L (1 +- (s- + s+) / (R- + R+)) exactly (from
 // R+^2 - R-^2 = s+^2 - s-^2), a sum of non-negative terms, so log1p((N - D)
 // / D) keeps full relative accuracy when the target is far from a short
-// piece; D is formed as d02 / (R - s) where R + s would cancel.  One
-// division.
-__device__ __forceinline__ double line_log(double sm, double sp, double Rm, double Rp, double d02, double L)
+// piece; D is formed as d02 / (R - s) where R + s would cancel.  The quotient
+// and the logarithm are one integer function of the five factors, and signs
+// are read from the bits: comparisons too would occupy the FP64 pipe.
+__device__ __forceinline__ double line_log(double sm, double sp, double Rm, double Rp, double d02, double L,
+                                           const NfTables& tab)
 {
     const double Sg = Rm + Rp, sg = sm + sp;
-    const double num = L * (Sg + fabs(sg));
-    const double a = (sg >= 0.0) ? Rm : Rp;
-    const double s = (sg >= 0.0) ? sm : -sp;
-    // selects, not branches: lanes see an edge from either side
-    const bool ahead = s >= 0.0;
-    const double numer = ahead ? num : num * (a - s);
-    const double denom = Sg * (ahead ? a + s : d02);
-    return log1p(numer / denom);
+    const bool behind = (nf_bits(sg) >> 63) != 0;
+    const double a = behind ? Rp : Rm;
+    const nf_u64 s = behind ? nf_bits(sp) ^ (1ull << 63) : nf_bits(sm);
+    const bool ahead = (s >> 63) == 0;
+    const double w = a + nf_double(s & 0x7fffffffffffffffull);
+    return nf_log1p_ratio(L, Sg + nf_double(nf_bits(sg) & 0x7fffffffffffffffull), ahead ? 1.0 : w, Sg,
+                          ahead ? w : d02, tab);
 }
 
 // A flat face in its own frame: origin x1, in-plane axes u (along the first
 // edge) and w = n x u, unit normal n; vertices at (0, 0), (L0, 0), (v3x,
 // v3y) (counter-clockwise about n); edge i runs from vertex i to i + 1 with
 // unit direction l_i (l_0 = (1, 0)) and length L_i; J = twice the area.
-// J = 0 marks a degenerate face.
+// J = 0 marks a degenerate face.  tol = NF_SNAP |x1|_1, the face's share of the
+// distances that count as zero.
 struct Face {
     double x1[3], u[3], w[3], n[3];
-    double J, L0, v3x, v3y, l1x, l1y, l2x, l2y, L1, L2;
+    double J, L0, v3x, v3y, l1x, l1y, l2x, l2y, L1, L2, tol, pad;
 };
 constexpr int FACE_DOUBLES = sizeof(Face) / sizeof(double);
-static_assert(FACE_DOUBLES == 22, "face record is 22 doubles");
+static_assert(FACE_DOUBLES == 24, "face record is 24 doubles");
 
 __device__ void make_face(V3 x1, V3 x2, V3 x3, Face& F)
 {
@@ -116,6 +127,8 @@ __device__ void make_face(V3 x1, V3 x2, V3 x3, Face& F)
     const double i1 = F.L1 > 0.0 ? 1.0 / F.L1 : 0.0, i2 = F.L2 > 0.0 ? 1.0 / F.L2 : 0.0;
     F.l1x = d1x * i1, F.l1y = d1y * i1;
     F.l2x = -F.v3x * i2, F.l2y = -F.v3y * i2;
+    F.tol = NF_SNAP * (fabs(x1.x) + fabs(x1.y) + fabs(x1.z));
+    F.pad = 0.0;
 }
 
 // One thread per face: kind 1 one face per triangle (its own vertex order),
@@ -175,12 +188,15 @@ __global__ void q2x_nearfield_faces(const NearArgs a, Face* faces)
 // write it, its determinant being -J h); the edge sum of the paper's form is
 // the same quantity as three atan pairs.  A target in the plane (h = 0 after
 // the snap) gets solid = 0, its direct value.
-__device__ __forceinline__ void face_potential(const Face* __restrict__ Fp, V3 r, double& single, double& solid,
-                                               double& h_out)
+// SINGLE false leaves out the logarithms (the double layer's value alone).
+// tol_r: the target's share of the distances that count as zero.
+template <bool SINGLE>
+__device__ __forceinline__ void face_potential(const Face* __restrict__ Fp, V3 r, double tol_r, const NfTables& tab,
+                                               double& single, double& solid, double& h_out)
 {
     const double J = __ldg(&Fp->J);
     single = solid = h_out = 0.0;
-    if (!(J > 0.0)) return;
+    if (nf_bits(J) == 0) return;  // J > 0 or exactly zero
     const V3 x1{__ldg(&Fp->x1[0]), __ldg(&Fp->x1[1]), __ldg(&Fp->x1[2])};
     const V3 d = sub(r, x1);
     const double rx = d.x * __ldg(&Fp->u[0]) + d.y * __ldg(&Fp->u[1]) + d.z * __ldg(&Fp->u[2]);
@@ -188,39 +204,56 @@ __device__ __forceinline__ void face_potential(const Face* __restrict__ Fp, V3 r
     double h = d.x * __ldg(&Fp->n[0]) + d.y * __ldg(&Fp->n[1]) + d.z * __ldg(&Fp->n[2]);
     // heights and in-plane distances below the rounding of the coordinates
     // are taken as zero: a target within that of the plane is in it
-    const double tol = NF_SNAP * (fabs(r.x) + fabs(r.y) + fabs(r.z) + fabs(x1.x) + fabs(x1.y) + fabs(x1.z));
-    if (fabs(h) <= tol) h = 0.0;
+    const nf_u64 tol = nf_bits(tol_r + __ldg(&Fp->tol));
+    const nf_u64 habs = nf_bits(h) & 0x7fffffffffffffffull;
+    const bool in_plane = habs <= tol;
+    if (in_plane) h = 0.0;
     const double h2 = h * h;
     const double L0 = __ldg(&Fp->L0), v3x = __ldg(&Fp->v3x), v3y = __ldg(&Fp->v3y);
-    // vertex offsets from the target's projection, and distances
-    const double ax = -rx, ay = -ry, bx = L0 - rx, by = -ry, cx = v3x - rx, cy = v3y - ry;
-    const double R1 = sqrt(ax * ax + ay * ay + h2), R2 = sqrt(bx * bx + by * by + h2),
-                 R3 = sqrt(cx * cx + cy * cy + h2);
-    const double lx[3] = {1.0, __ldg(&Fp->l1x), __ldg(&Fp->l2x)};
-    const double ly[3] = {0.0, __ldg(&Fp->l1y), __ldg(&Fp->l2y)};
-    const double Ls[3] = {L0, __ldg(&Fp->L1), __ldg(&Fp->L2)};
-    const double px[4] = {ax, bx, cx, ax}, py[4] = {ay, by, cy, ay};
-    const double Rv[4] = {R1, R2, R3, R1};
+    // vertex offsets from the target's projection: (-rx, -ry), (bx, -ry),
+    // (cx, cy), and distances
+    const double bx = L0 - rx, cx = v3x - rx, cy = v3y - ry;
+    const double q = fma(ry, ry, h2), qc = fma(-ry, cy, h2);
+    const double R1 = nf_sqrt(fma(rx, rx, q)), R2 = nf_sqrt(fma(bx, bx, q)),
+                 R3 = nf_sqrt(fma(cx, cx, fma(cy, cy, h2)));
     double S = 0.0;
+    if (SINGLE) {
+        const double lx[3] = {1.0, __ldg(&Fp->l1x), __ldg(&Fp->l2x)};
+        const double ly[3] = {0.0, __ldg(&Fp->l1y), __ldg(&Fp->l2y)};
+        const double Ls[3] = {L0, __ldg(&Fp->L1), __ldg(&Fp->L2)};
+        const double px[3] = {-rx, bx, cx}, py[3] = {-ry, -ry, cy};
+        const double Rv[4] = {R1, R2, R3, R1};
 #pragma unroll
-    for (int i = 0; i < 3; ++i) {
-        const double sm = px[i] * lx[i] + py[i] * ly[i];
-        const double sp = px[i + 1] * lx[i] + py[i + 1] * ly[i];
-        double t = px[i] * ly[i] - py[i] * lx[i];  // offset . m_i, m_i = (l_y, -l_x) the outward normal
-        if (fabs(t) <= tol) t = 0.0;                // target on the edge's line
-        if (t != 0.0 && Ls[i] > 0.0) S += t * line_log(sm, sp, Rv[i], Rv[i + 1], t * t + h2, Ls[i]);
+        for (int i = 0; i < 3; ++i) {
+            // the edge's ends along it, and offset . m_i, m_i = (l_y, -l_x) the outward normal
+            const double sm = i ? px[i] * lx[i] + py[i] * ly[i] : -rx;
+            const double sp = i ? sm + Ls[i] : bx;
+            const double t = i ? px[i] * ly[i] - py[i] * lx[i] : ry;
+            if ((nf_bits(t) & 0x7fffffffffffffffull) > tol && nf_bits(Ls[i]) != 0)  // else on the edge's line
+                S += t * line_log(sm, sp, Rv[i], Rv[i + 1], fma(t, t, h2), Ls[i], tab);
+        }
     }
-    if (h != 0.0) {
-        const double den = R1 * R2 * R3 + (ax * bx + ay * by + h2) * R3 + (ax * cx + ay * cy + h2) * R2 +
-                           (bx * cx + by * cy + h2) * R1;
-        solid = 2.0 * atan2(J * h, den);
+    if (!in_plane) {
+        const double den = fma(R3, fma(R1, R2, fma(-rx, bx, q)), fma(fma(-rx, cx, qc), R2, fma(bx, cx, qc) * R1));
+        const double om = nf_atan2(J * nf_double(habs), den, tab);
+        solid = nf_double(nf_bits(om + om) | (nf_bits(h) & (1ull << 63)));
     }
     single = S - h * solid;
     h_out = h;
 }
 
-__global__ void q2x_nearfield_kernel(const NearArgs a, const Face* __restrict__ faces)
+template <int KIND, int LAYER>
+__global__ void __launch_bounds__(128) q2x_nearfield_kernel(const NearArgs a, const Face* __restrict__ faces)
 {
+    __shared__ unsigned s_k[256];
+    __shared__ nf_u64 s_log[256], s_atan[65];
+    for (int i = threadIdx.x; i < 256; i += 128) {
+        s_k[i] = nf_log_k[i];
+        s_log[i] = nf_log_t[i];
+        if (i < 65) s_atan[i] = nf_atan_t[i];
+    }
+    __syncthreads();
+    const NfTables tab{s_k, s_log, s_atan};
     const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= a.n_tgt) return;
     int64_t j0 = __ldg(a.tgt_off + t), j1 = __ldg(a.tgt_off + t + 1);
@@ -229,6 +262,7 @@ __global__ void q2x_nearfield_kernel(const NearArgs a, const Face* __restrict__ 
         j0 = j1 = 0;
     }
     const V3 r{__ldg(a.tgt + t), __ldg(a.tgt + a.n_tgt + t), __ldg(a.tgt + 2 * a.n_tgt + t)};
+    const double tol_r = NF_SNAP * (fabs(r.x) + fabs(r.y) + fabs(r.z));
     double acc = 0.0;
 #pragma unroll 1
     for (int64_t j = j0; j < j1; ++j) {
@@ -238,7 +272,7 @@ __global__ void q2x_nearfield_kernel(const NearArgs a, const Face* __restrict__ 
             continue;
         }
         double val = 0.0;
-        if (a.kind == 0) {  // segment
+        if constexpr (KIND == 0) {  // segment
             const int64_t v0 = __ldg(a.idx + e), v1 = __ldg(a.idx + a.n_elem + e);
             if (v0 < 0 || v0 >= a.n_vert || v1 < 0 || v1 >= a.n_vert) {
                 atomicOr(a.err, 1u);
@@ -247,22 +281,22 @@ __global__ void q2x_nearfield_kernel(const NearArgs a, const Face* __restrict__ 
             const V3 X0{__ldg(a.vx + v0), __ldg(a.vy + v0), __ldg(a.vz + v0)};
             const V3 X1{__ldg(a.vx + v1), __ldg(a.vy + v1), __ldg(a.vz + v1)};
             const V3 ev = sub(X1, X0);
-            const double L = sqrt(dot(ev, ev));
+            const double L = nf_sqrt(dot(ev, ev));
             if (L > 0.0) {
                 const V3 l = scale(ev, 1.0 / L);
                 const V3 pa = sub(X0, r), pb = sub(X1, r);
                 const V3 c = cross(pa, l);
-                val = line_log(dot(pa, l), dot(pb, l), sqrt(dot(pa, pa)), sqrt(dot(pb, pb)), dot(c, c), L);
+                val = line_log(dot(pa, l), dot(pb, l), nf_sqrt(dot(pa, pa)), nf_sqrt(dot(pb, pb)), dot(c, c), L, tab);
             }
-        } else if (a.kind == 1) {  // triangle
+        } else if constexpr (KIND == 1) {  // triangle
             double single, solid, h;
-            face_potential(faces + e, r, single, solid, h);
-            val = a.layer ? solid : single;
+            face_potential<LAYER == 0>(faces + e, r, tol_r, tab, single, solid, h);
+            val = LAYER ? solid : single;
         } else {  // tetrahedron: -1/2 sum over the outward faces of h_f int_f 1/|r - y| dS
 #pragma unroll 1
             for (int f = 0; f < 4; ++f) {
                 double single, solid, h;
-                face_potential(faces + 4 * e + f, r, single, solid, h);
+                face_potential<true>(faces + 4 * e + f, r, tol_r, tab, single, solid, h);
                 val -= 0.5 * h * single;
             }
         }
@@ -321,7 +355,15 @@ extern "C" q2x_status q2x_nearfield(q2x_plan_t plan, int kind, int layer, int64_
         if (e != cudaSuccess) return q2x_cuda_fail(plan, e, "q2x_nearfield_faces launch");
         plan->launches += 1;
     }
-    q2x::q2x_nearfield_kernel<<<(unsigned)((n_tgt + 127) / 128), 128, 0, plan->stream>>>(a, faces);
+    const unsigned grid = (unsigned)((n_tgt + 127) / 128);
+    if (kind == 0)
+        q2x::q2x_nearfield_kernel<0, 0><<<grid, 128, 0, plan->stream>>>(a, faces);
+    else if (kind == 1 && layer == 0)
+        q2x::q2x_nearfield_kernel<1, 0><<<grid, 128, 0, plan->stream>>>(a, faces);
+    else if (kind == 1)
+        q2x::q2x_nearfield_kernel<1, 1><<<grid, 128, 0, plan->stream>>>(a, faces);
+    else
+        q2x::q2x_nearfield_kernel<2, 0><<<grid, 128, 0, plan->stream>>>(a, faces);
     e = cudaGetLastError();
     if (e != cudaSuccess) return q2x_cuda_fail(plan, e, "q2x_nearfield_kernel launch");
     plan->launches += 1;
