@@ -611,6 +611,53 @@ q2x_status q2x_plan_workspace(q2x_plan_t plan, size_t bytes)
     return ensure_ws(plan, bytes);
 }
 
+q2x_status q2x_galerkin_directions(q2x_plan_t plan, int64_t n_elem, int64_t n_vert, const double* vxyz,
+                                   const int32_t* idx, const double* sigma, int64_t n_leaves, const int64_t* leaf_off,
+                                   const double* leaf_c, int layer, const double* w, double* out, bool* taken)
+{
+    const int p = plan->p_max, np = (p + 1) * (p + 1);
+    const q2x::DirShape shape = q2x::dir_shape(p, 1, n_elem, n_leaves);
+    const size_t bytes = leaf_tile_ws_bytes(n_elem, n_leaves, np, shape.T, 0);
+    *taken = n_leaves < ((int64_t)1 << 31) && bytes <= ((size_t)8 << 30);
+    if (!*taken) return Q2X_OK;
+    q2x_status st = ensure_ws(plan, bytes);
+    if (st != Q2X_OK) return st;
+    q2x::DirArgs a{};
+    a.p_max = p;
+    cudaError_t e = q2x::dir_setup(a, q2x::KIND_TRI, Q2X_DENSITY_CONST, shape.nt);
+    if (e != cudaSuccess) return cuda_fail(plan, e, "direction tables");
+    q2x::LeafTileWork lw;
+    leaf_tile_carve(static_cast<unsigned char*>(plan->ws), n_elem, n_leaves, np, shape.T, 0, lw, nullptr);
+    lw.max_slots = (int64_t)1 << 62;  // tiles keep no partial rows here: none is dropped for want of one
+    e = q2x::leaf_tiles_build(leaf_off, n_leaves, shape.T, 0, 0, lw, plan->stream);
+    if (e == cudaSuccess) e = cudaMemsetAsync(lw.counter, 0, sizeof(unsigned long long), plan->stream);
+    if (e != cudaSuccess) return cuda_fail(plan, e, "leaf tile list");
+    a.kind = q2x::BatchKind{n_elem, n_vert, vxyz, vxyz + n_vert, vxyz + 2 * n_vert, idx, sigma};
+    a.n_leaves = n_leaves;
+    a.leaf_c = leaf_c;
+    a.np = np;
+    a.norm = plan->norm;
+    a.tiles = lw.tiles;
+    a.n_tiles_dev = lw.n_tiles;
+    a.counter = lw.counter;
+    a.gal_w = w;
+    a.gal_out = out;
+    a.err = plan->d_err;
+    const int combo = layer ? 10 : 9;
+    const q2x::DirFns& f = q2x::dir_fns(shape.cls, combo);
+    int& occ = plan->dir_occ[shape.nt / 32][combo];
+    if (occ == 0) {
+        e = f.occupancy(&occ, p, shape.nt, shape.T);
+        if (e != cudaSuccess) return cuda_fail(plan, e, "direction kernel occupancy query");
+        if (occ <= 0) return fail(plan, Q2X_ERR_CUDA, "direction kernel does not fit on the device");
+    }
+    const int64_t grid = std::min<int64_t>((int64_t)occ * plan->num_sms, lw.max_tiles);
+    e = f.launch(a, shape.nt, shape.T, (int)grid, plan->stream);
+    if (e != cudaSuccess) return cuda_fail(plan, e, "direction kernel launch");
+    plan->launches += 4;
+    return Q2X_OK;
+}
+
 extern "C" {
 
 q2x_status q2x_plan(q2x_plan_t* out, int p_max, q2x_norm norm, q2x_precision precision,

@@ -43,13 +43,14 @@ cudaError_t dir_occupancy(int* blocks, int p, int nt, int T)
      Q2X_DIR_FNS(KIND_TRI, DENS_CONST, 2, M),  Q2X_DIR_FNS(KIND_TRI, DENS_CONST, 3, M),                      \
      Q2X_DIR_FNS(KIND_TRI, DENS_LINEAR, 1, M), Q2X_DIR_FNS(KIND_TRI, DENS_LINEAR, 2, M),                     \
      Q2X_DIR_FNS(KIND_TRI, DENS_LINEAR, 3, M), Q2X_DIR_FNS(KIND_TET, DENS_CONST, 1, M),                      \
-     Q2X_DIR_FNS(KIND_SEG, DENS_CONST, 4, M)}
+     Q2X_DIR_FNS(KIND_SEG, DENS_CONST, 4, M),  Q2X_DIR_FNS(KIND_TRI, DENS_CONST, 9, M),                      \
+     Q2X_DIR_FNS(KIND_TRI, DENS_CONST, 10, M)}
 
 }  // namespace
 
 const DirFns& dir_fns(int cls, int combo)
 {
-    static const DirFns f[2][9] = {Q2X_DIR_ROW(256), Q2X_DIR_ROW(128)};
+    static const DirFns f[2][11] = {Q2X_DIR_ROW(256), Q2X_DIR_ROW(128)};
     return f[cls][combo];
 }
 

@@ -205,6 +205,8 @@ struct DirArgs {
     const int64_t* n_tiles_dev;
     unsigned long long* counter;
     const double* wvec;  // vector density: SoA 3 x n_elem components per element
+    const double* gal_w; // receiver side: weights [n_leaves][np] of the packed columns,
+    double* gal_out;     // and its results [n_elem]
     double* partial[3];
     double* coef[3];
     unsigned* err;
@@ -220,6 +222,8 @@ struct DirCfg {
     static constexpr bool DBL = KIND == KIND_TRI && (OUTS & 2) != 0;
     // a vector density: unit-density values, three weighted sums
     static constexpr bool VEC = (OUTS & 4) != 0;
+    // receiver side: each element's own value against weights (one layer)
+    static constexpr bool GAL = (OUTS & 8) != 0;
     static constexpr bool SGL = (OUTS & 1) != 0 || VEC;
     static constexpr int NL = KIND + 2 + (LIN ? 2 : 0);  // q, p | j, i | b, a; linear: q, j, E, i, Iw
     // what the stored values of level k carry, in units of 2^32 (mul2)
@@ -234,13 +238,191 @@ struct DirCfg {
         const size_t a = (size_t)T * REC * 8, s = (size_t)(p + 1) * 2 * (p + 1) * LAYERS * 8;
         return ((a > s ? a : s) + 15) / 16 * 16;
     }
+    // receiver side: the fixed-point weights [degree][direction] (16 bytes), the
+    // scaled column weights (8) and products (8) they come from, and the
+    // elements' values per direction [element][direction]
+    __host__ __device__ static constexpr size_t gal_bytes(int p)
+    {
+        return (size_t)(p + 1) * (p + 1) * 40 + 16;
+    }
     __host__ __device__ static constexpr size_t smem(int p, int T, int nt)
     {
+        if (GAL) return (size_t)(p + 1) * 48 + ((size_t)T * REC * 8 + 15) / 16 * 16 + gal_bytes(p) + (size_t)T * (p + 1) * 8;
         return (size_t)(p + 1) * 48 + rec_bytes(p, T) + (size_t)LAYERS * (p + 1) * nt * 16;
     }
 };
 
 __device__ __forceinline__ Fx as_fx(int2 v) { return Fx{v.x, v.y}; }
+
+// Receiver side: out[e] = sum_c w_c P_c(e) over the packed columns c of an
+// element's own coefficients.  The weights are carried to the directions
+// (the transposed map, exact products per degree), and sum_n W_n h_n(u1, u2,
+// u3) of the chain's values h is nested Horner steps from the highest degree
+// down, one per level and degree:
+//   c_n = W_n + u1 c_{n+1}, b_n = c_n + u3 b_{n+1}, a_n = b_n + u2 a_{n+1},
+// the value a_0 (double layer: of the weights one degree up, times the
+// normal's multiplier).  The weights are scaled so that the bound of all
+// partial sums is 2^59.
+template <typename D>
+__device__ __forceinline__ void dir_gal_tile(const DirArgs& a, int T, const BatchTile& t, int n_el, int kr, int ex,
+                                             int Ej, const int2* rec, const int2* dirs, int g, int j)
+{
+    constexpr bool DBL = D::DBL;
+    const int tid = threadIdx.x, lane = tid & 31, NT = blockDim.x;
+    const int J = a.J, p = a.p_max, np = a.np;
+    unsigned char* base = reinterpret_cast<unsigned char*>(const_cast<int2*>(rec)) + ((size_t)T * D::REC * 8 + 15) / 16 * 16;
+    longlong2* W = reinterpret_cast<longlong2*>(base);                       // [p + 1][J]
+    long long* prod = reinterpret_cast<long long*>(W + (p + 1) * J);         // [p + 1][2 J]
+    int2* col = reinterpret_cast<int2*>(prod + (p + 1) * 2 * J);             // [np]
+    long long* val = reinterpret_cast<long long*>(base + D::gal_bytes(p));   // [T][J]
+    __shared__ int s_e[Q2X_P_MAX + 1], s_scale;
+    __shared__ double s_sum[Q2X_P_MAX + 1];
+    constexpr int d = DBL ? KIND_TRI : KIND_TRI + 1;
+    const double* w = a.gal_w + (int64_t)t.leaf * np;
+    for (int n = tid >> 5; n <= p; n += NT >> 5) {
+        const int ns = DBL ? n - 1 : n;  // the frame's power
+        const double fr = ns > 0 ? __ldg(a.pw + (kr + 7) * 24 + ns) : 1.0;
+        double v[2] = {0.0, 0.0};
+        int top = 0;
+#pragma unroll
+        for (int c = 0; c < 2; ++c) {
+            const int q = lane + 32 * c;
+            if (q <= 2 * n && !(DBL && n == 0)) {
+                const int k = n * n + q;
+                v[c] = __ldg(w + k) * __ldg(a.col + (a.norm * 4 + d) * 441 + k) * fr;
+                if ((col_desc(k) >> (5 + a.norm)) & 1) v[c] = -v[c];
+                top = max(top, hi32(__double_as_longlong(v[c])) & 0x7fffffff);
+            }
+        }
+        top = __reduce_max_sync(0xffffffffu, top);
+        const int e1 = max(top >> 20, 1);
+#pragma unroll
+        for (int c = 0; c < 2; ++c) {
+            const int q = lane + 32 * c;
+            if (q <= 2 * n) {
+                const long long x = top < 0x7ff00000 ? dir_fixed((unsigned long long)__double_as_longlong(v[c]), e1, 56) : 0;
+                const int h = (int)((x + (1ll << 27)) >> 28);
+                col[n * n + q] = make_int2(h, (int)(x - ((long long)h << 28)));
+            }
+        }
+        __syncwarp();
+        double sum = 0.0;
+#pragma unroll
+        for (int c = 0; c < 2; ++c) {
+            const int s = lane + 32 * c;
+            if (s < 2 * J) {
+                long long hh = 0, mid = 1ll << 27;
+                const int2* P = a.inv + s * np + n * n;
+#pragma unroll 4
+                for (int q = 0; q <= 2 * n; ++q) {
+                    const int2 m = __ldg(P + q), x = col[n * n + q];
+                    mid = madw(m.x, x.y, mid);
+                    mid = madw(m.y, x.x, mid);
+                    hh = madw(m.x, x.x, hh);
+                }
+                hh += mid >> 28;
+                prod[n * 2 * J + s] = hh;
+                sum += fabs((double)hh);
+            }
+        }
+        for (int o = 16; o; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+        if (lane == 0) {
+            // (weights beyond FP64 make the tile's results NaN)
+            s_sum[n] = top < 0x7ff00000 ? sum * (DBL ? 0.5 * n * (n + 1) : 0.5 * (n + 1) * (n + 2))
+                                        : __longlong_as_double(0x7ff0000000000000ll);
+            s_e[n] = e1 - 1022 - 58 + (ns > 0 ? ns * (ex - 1022) : 0);
+        }
+    }
+    __syncthreads();
+    if (tid == 0) {
+        int most = -1000000;
+        for (int n = 0; n <= p; ++n)
+            if (s_sum[n] > 0.0) most = max(most, s_e[n] + (hi32(__double_as_longlong(s_sum[n])) >> 20) - 1022);
+        double B = 0.0;
+        for (int n = 0; n <= p; ++n) B += s_sum[n] * pow2d(max(s_e[n] - most, -1000));
+        int scale = 0;
+        if (B > 0.0) scale = 59 - (most + (hi32(__double_as_longlong(B)) >> 20) - 1022);
+        s_scale = B < 1e300 ? scale : 0x7fffffff;
+    }
+    __syncthreads();
+    const int scale = s_scale;
+    for (int i = tid; i < (p + 1) * J; i += NT) {
+        const int n = i / J, jj = i - n * J;
+        const int sh = scale == 0x7fffffff ? -100 : s_e[n] + scale;
+        auto put = [&](long long v) {
+            if (sh >= 0) return v << min(sh, 62);
+            if (sh < -62) return 0ll;
+            return (v + (1ll << (-sh - 1))) >> -sh;
+        };
+        longlong2 o;
+        o.x = put(prod[n * 2 * J + 2 * jj]);
+        o.y = -put(prod[n * 2 * J + 2 * jj + 1]);
+        W[i] = o;
+    }
+    __syncthreads();
+    const long long rnd = a.rnd;
+    if (g < a.G) {
+#pragma unroll 1
+        for (int e = g; e < n_el; e += a.G) {
+            const int2* r = rec + e * D::REC;
+            Mul u[3], nu{};
+            {
+                Fx da[6];
+#pragma unroll
+                for (int c = 0; c < 6; ++c) da[c] = as_fx(dirs[j * 6 + c]);
+#pragma unroll
+                for (int k = 0; k < 3; ++k) {
+                    const Fx y[3] = {as_fx(r[3 * k]), as_fx(r[3 * k + 1]), as_fx(r[3 * k + 2])};
+                    u[k] = mul_of(dir_dot(da, y, rnd), dir_dot(da + 3, y, rnd));
+                }
+                if (DBL) {
+                    const Fx y[3] = {as_fx(r[D::R_NRM]), as_fx(r[D::R_NRM + 1]), as_fx(r[D::R_NRM + 2])};
+                    nu = mul_of(dir_dot(da, y, rnd), dir_dot(da + 3, y, rnd));
+                }
+            }
+            long long res = 0;
+            if (!DBL || p > 0) {
+                const longlong2* q = W + p * J + j;
+                longlong2 w0 = *q;
+                Cx c{w0.x + dir_bias(1), w0.y + dir_bias(1)}, b{w0.x + dir_bias(2), w0.y + dir_bias(2)},
+                    x{w0.x + dir_bias(3), w0.y + dir_bias(3)};
+                CxH hc = high_of<1>(c), hb = high_of<2>(b), hx = high_of<3>(x);
+#pragma unroll 4
+                for (int n = p - 1; n >= (DBL ? 1 : 0); --n) {
+                    q -= J;
+                    w0 = *q;
+                    c = mul_add<true>(u[0], c, hc, Cx{w0.x, w0.y}, rnd);
+                    hc = high_of<1>(c);
+                    b = mul_add<true>(u[2], b, hb, c, rnd);
+                    hb = high_of<2>(b);
+                    x = mul_add<true>(u[1], x, hx, b, rnd);
+                    hx = high_of<3>(x);
+                }
+                if (DBL)
+                    res = mul2<false>(nu.rh, nu.rl, nu.nh, nu.nl, (int)x.re, hx.rh, (int)x.im, hx.ih, 0, rnd) - dir_bias(1);
+                else
+                    res = x.re - dir_bias(3);
+            }
+            val[e * J + j] = res;
+        }
+    }
+    __syncthreads();
+    if (tid < n_el) {
+        long long sum = 0;
+        for (int k = 0; k < J; ++k) sum += val[tid * J + k];
+        const int2 sd = rec[tid * D::REC + D::R_SEED];
+        double v = (double)sum * __longlong_as_double(((long long)sd.y << 32) | (unsigned)sd.x);
+        int e2 = -scale + (DBL ? 1 : 0) + (KIND_TRI + 1) * Ej;  // (half the normal)
+        if (e2 > 1000 || e2 < -1000) {
+            const int h = max(-2000, min(2000, e2)) / 2;
+            v *= pow2d(h);
+            e2 = max(-2000, min(2000, e2)) - h;
+        }
+        v *= pow2d(e2);
+        if (scale == 0x7fffffff) v = __longlong_as_double(0x7ff8000000000000ll);
+        a.gal_out[t.e_lo + tid] = v;
+    }
+}
 
 // MAX_NT 256: two CTAs of up to 128 registers a thread; 128: six of up to 80.
 template <int KIND, int DENS, int OUTS, int MAX_NT>
@@ -249,7 +431,7 @@ __global__ void __launch_bounds__(MAX_NT, MAX_NT == 256 ? 2 : 6) q2x_dir_kernel(
     using D = DirCfg<KIND, DENS, OUTS>;
     constexpr int NV = D::NV;
     constexpr int NL = D::NL;
-    constexpr bool LIN = D::LIN, DBL = D::DBL, SGL = D::SGL, VEC = D::VEC;
+    constexpr bool LIN = D::LIN, DBL = D::DBL, SGL = D::SGL, VEC = D::VEC, GAL = D::GAL;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int tid = threadIdx.x, NT = blockDim.x;
     const int J = a.J, G = a.G, np = a.np;
@@ -459,11 +641,18 @@ __global__ void __launch_bounds__(MAX_NT, MAX_NT == 256 ? 2 : 6) q2x_dir_kernel(
                     r[D::R_DENS + k] = make_int2(f.h, f.l);
                 }
             }
-            const long long sd =
-                (live && wmax < 0x7ff00000) ? dir_fixed((unsigned long long)__double_as_longlong(w), ew, a.seed_bits) : 0;
+            long long sd = 0;
+            if (GAL)  // the factor of the element's value
+                sd = live ? __double_as_longlong(w) : over ? 0x7ff8000000000000ll : 0;
+            else if (live && wmax < 0x7ff00000)
+                sd = dir_fixed((unsigned long long)__double_as_longlong(w), ew, a.seed_bits);
             r[D::R_SEED] = make_int2((int)sd, hi32(sd));
         }
         __syncthreads();
+        if constexpr (GAL) {
+            dir_gal_tile<D>(a, T, t, n_el, kr, ex, Ej, rec, dirs, g, j);
+            continue;
+        }
 
         // ---- the recurrences: this thread's direction, elements g, g + G, ..
         if (g < G) {
@@ -708,7 +897,8 @@ struct DirFns {
 };
 // [CTA class: 0 up to 256 threads, 1 up to 128][combo]; combos: 0 segments, 1-3
 // triangles constant density (single, double, both), 4-6 linear density, 7
-// tetrahedra, 8 segments carrying a vector density (the element kernel's order)
+// tetrahedra, 8 segments carrying a vector density (the element kernel's
+// order), 9 and 10 the receiver side, single layer and normal derivative
 const DirFns& dir_fns(int cls, int combo);
 // A call's CTAs: class, threads, elements per tile.
 struct DirShape {

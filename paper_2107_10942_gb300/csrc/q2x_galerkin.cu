@@ -14,6 +14,10 @@
 // each lane contracts its own element's staged row with the leaf's weights,
 // which a first kernel folds together with the per-column finish constants
 // (1/(n+d)!, the packing sign, 1/4pi, the leaf's power-of-two scale).  FP64.
+//
+// Calls run by directions in fixed point (dir_gal_tile in q2x_dir.cuh, on the
+// integer pipe); the kernel here, bound by the FP64 pipe, is left for leaf
+// lists whose tiles would not fit the workspace bound.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -131,7 +135,11 @@ extern "C" q2x_status q2x_galerkin_triangles(q2x_plan_t plan, int64_t n_elem, in
     if (e != cudaSuccess) return q2x_cuda_fail(plan, e, "cudaSetDevice");
     const int p = plan->p_max;
     const int np = (p + 1) * (p + 1);
-    q2x_status st = q2x_plan_workspace(plan, sizeof(double) * (size_t)n_leaves * np);
+    bool taken = false;
+    q2x_status st = q2x_galerkin_directions(plan, n_elem, n_vert, vxyz, idx, sigma, n_leaves, leaf_off, leaf_c, layer, w,
+                                            out, &taken);
+    if (st != Q2X_OK || taken) return st;
+    st = q2x_plan_workspace(plan, sizeof(double) * (size_t)n_leaves * np);
     if (st != Q2X_OK) return st;
     double* wf = static_cast<double*>(plan->ws);
     using C = q2x::Chain<q2x::KIND_TRI, q2x::DENS_CONST>;

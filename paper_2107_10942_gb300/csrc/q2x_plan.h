@@ -22,7 +22,7 @@ struct q2x_plan_s {
     size_t ws_bytes = 0;
     int occ_cache[2][9][5] = {};  // [precision][element combo][capacity bin]
     int tile_occ[4][5] = {};  // resident CTAs per SM of the FP32 leaf-tile kernels [combo][bin]
-    int dir_occ[9][9] = {};  // resident CTAs per SM of the FP64 direction kernels [warps per CTA][combo]
+    int dir_occ[9][11] = {};  // resident CTAs per SM of the FP64 direction kernels [warps per CTA][combo]
     int timing = 0;
     std::vector<cudaEvent_t> ev_pool;                            // idle events
     std::vector<std::pair<cudaEvent_t, cudaEvent_t>> ev_pending;  // recorded pairs
@@ -36,3 +36,8 @@ q2x_status q2x_cuda_fail(q2x_plan_t plan, cudaError_t e, const char* what);
 // grow the plan's device workspace to at least `bytes` (synchronises the
 // plan's stream when it has to reallocate)
 q2x_status q2x_plan_workspace(q2x_plan_t plan, size_t bytes);
+// Receiver-side integration by the direction kernels (q2x_api.cu): *taken
+// false where the call has to take the row kernel (its tile list would not fit).
+q2x_status q2x_galerkin_directions(q2x_plan_t plan, int64_t n_elem, int64_t n_vert, const double* vxyz,
+                                   const int32_t* idx, const double* sigma, int64_t n_leaves, const int64_t* leaf_off,
+                                   const double* leaf_c, int layer, const double* w, double* out, bool* taken);

@@ -172,3 +172,40 @@ def _degree_max(a, p):
     for n in range(p + 1):
         out[:, n * n:(n + 1) ** 2] = a[:, n * n:(n + 1) ** 2].max(axis=1, keepdims=True)
     return out
+
+
+@pytest.mark.parametrize("layer", [0, 1])
+@pytest.mark.parametrize("small", [True, False])
+@pytest.mark.parametrize("p", [0, 1, 4, 12, 17, 20])
+def test_galerkin_side(q2x, p, small, layer):
+    """Receiver-side integrals against per-element rows contracted on the host,
+    weights of all degrees of one size in the scaled norm."""
+    import torch
+    prob = random_problem("triangle", edge_sizes(p, small), seed=p + 70, p=p)
+    rng = np.random.default_rng(p)
+    leaf_of = np.repeat(np.arange(len(prob["leaf_off"]) - 1), np.diff(prob["leaf_off"]))
+    w = rng.standard_normal((prob["leaf_c"].shape[1], (p + 1) ** 2)) * _scales(p) / prob["leaf_rho"][:, None] ** _degree(p)
+    t = lambda x: torch.from_numpy(np.ascontiguousarray(x)).cuda()
+    d = {k: t(v) for k, v in prob.items() if hasattr(v, "dtype")}
+    plan = q2x.Plan(p, norm="moment")
+    got = plan.galerkin_triangles(d["vxyz"], d["idx"], t(w), d["leaf_off"], d["leaf_c"], d["leaf_rho"], d["sigma"],
+                                  layer=layer).cpu().numpy()
+    rows = plan.triangles(d["vxyz"], d["idx"], d["sigma"], None, t(prob["leaf_c"][:, leaf_of]),
+                          t(prob["leaf_rho"][leaf_of]), single=layer == 0, double=layer == 1)[layer].cpu().numpy()
+    plan.sync()
+    terms = rows * w[leaf_of]
+    # both sides round every column's term to some (p + 1) units of 2^-53 of its bound: the
+    # degree's largest weight times the element's largest scaled row entry, 2n + 1 columns
+    size = np.abs(w * prob["leaf_rho"][:, None] ** _degree(p) / _scales(p)).max(1)[leaf_of] * np.abs(
+        rows / prob["leaf_rho"][leaf_of][:, None] ** _degree(p) * _scales(p)).max(1)
+    assert np.all(np.abs(got - terms.sum(1)) <= 1e-13 * (p + 1) ** 2 * np.maximum(size, 1e-300))
+
+
+def _degree(p):
+    return np.concatenate([np.full(2 * n + 1, float(n)) for n in range(p + 1)])
+
+
+def _scales(p):
+    import math
+    return np.array([math.sqrt(math.factorial(n + abs(m)) * math.factorial(n - abs(m)))
+                     for n in range(p + 1) for m in range(-n, n + 1)])
