@@ -139,20 +139,6 @@ int bin_index(int p)
 
 // ------------------------------------------------------------ small kernels
 
-// leaf_off must be non-decreasing with leaf_off[0] = 0, leaf_off[n_leaves] = n_elem
-__global__ void check_leaf_off_kernel(const int64_t* off, int64_t n_leaves, int64_t n_elem,
-                                      unsigned* err)
-{
-    const int64_t L = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (L > n_leaves) return;
-    const int64_t o = off[L];
-    bool bad = (o < 0 || o > n_elem);
-    if (L == 0 && o != 0) bad = true;
-    if (L == n_leaves && o != n_elem) bad = true;
-    if (L < n_leaves && off[L + 1] < o) bad = true;
-    if (bad) atomicOr(err, Q2X_DEVERR_LEAF_OFF);
-}
-
 // per-leaf scale: largest distance from the centre to a vertex of its
 // elements, as the bit pattern of a non-negative float (atomicMax on ints
 // orders non-negative floats correctly)
@@ -197,7 +183,7 @@ __global__ void leaf_reduce_kernel(const double* __restrict__ elem, int np, int6
     const int64_t L = unit / np;
     if (L >= n_leaves) return;
     const int c = (int)(unit - L * np);
-    // clamped: a bad leaf_off is reported by check_leaf_off_kernel, never read past
+    // clamped: a bad leaf_off is reported by check_leaf_off, never read past
     const int64_t e0 = min(max(off[L], (int64_t)0), n_elem);
     const int64_t e1 = min(max(off[L + 1], e0), n_elem);
     const double* col = elem + c;
@@ -318,10 +304,8 @@ q2x_status run_directions(q2x_plan_t plan, q2x::DirArgs& a, int combo, const q2x
     q2x::LeafTileWork w;
     double* partial[3] = {nullptr, nullptr, nullptr};
     leaf_tile_carve(static_cast<unsigned char*>(plan->ws), n_elem, n_leaves, np, shape.T, layers, w, partial);
-    const int64_t nb = (n_leaves + 1 + 255) / 256;
-    check_leaf_off_kernel<<<(unsigned)nb, 256, 0, plan->stream>>>(leaf_off, n_leaves, n_elem, plan->d_err);
-    cudaError_t e = q2x::leaf_tiles_build(leaf_off, n_leaves, shape.T, 0, 0, w, plan->stream);
-    if (e == cudaSuccess) e = cudaMemsetAsync(w.counter, 0, sizeof(unsigned long long), plan->stream);
+    int built = 0;
+    cudaError_t e = q2x::leaf_tiles_build(leaf_off, n_leaves, shape.T, 0, 0, w, plan->d_err, &built, plan->stream);
     if (e != cudaSuccess) return cuda_fail(plan, e, "leaf tile list");
     a.kind = q2x::BatchKind{n_elem, n_vert, vxyz, vxyz + n_vert, vxyz + 2 * n_vert, idx, sigma};
     a.n_leaves = n_leaves;
@@ -364,7 +348,7 @@ q2x_status run_directions(q2x_plan_t plan, q2x::DirArgs& a, int combo, const q2x
         if (out[l])
             e = q2x::leaf_tiles_combine(partial[l], w.slot_off, leaf_off, np, n_leaves, out[l], accumulate, plan->stream);
     if (e != cudaSuccess) return cuda_fail(plan, e, "leaf tile combine");
-    plan->launches += 5 + layers;
+    plan->launches += built + 1 + layers;
     return Q2X_OK;
 }
 
@@ -443,7 +427,7 @@ q2x_status run_elements(q2x_plan_t plan, int kind, int dens, int64_t n_elem, int
     const bool dirs = prec == 0 && leaf_off && n_leaves < ((int64_t)1 << 31);
     q2x::DirArgs da{};
     const int dir_layers = vec ? 3 : (coef0 ? 1 : 0) + (dbl ? 1 : 0);
-    const q2x::DirShape shape = q2x::dir_shape(plan->p_max, dir_layers, n_elem, n_leaves);
+    const q2x::DirShape shape = q2x::dir_shape(plan->p_max, dir_layers, n_elem, n_leaves, plan->num_sms);
     size_t dir_bytes = 0;
     if (dirs) {
         da.p_max = plan->p_max;
@@ -474,9 +458,9 @@ q2x_status run_elements(q2x_plan_t plan, int kind, int dens, int64_t n_elem, int
     if (st != Q2X_OK) return st;
     unsigned char* ws = static_cast<unsigned char*>(plan->ws);
 
-    if (leaf_off) {
-        const int64_t nb = (n_leaves + 1 + 255) / 256;
-        check_leaf_off_kernel<<<(unsigned)nb, 256, 0, plan->stream>>>(leaf_off, n_leaves, n_elem, plan->d_err);
+    if (leaf_off && !tiles) {  // (the tile list's build checks it too)
+        e = q2x::check_leaf_off(leaf_off, n_leaves, n_elem, plan->d_err, plan->stream);
+        if (e != cudaSuccess) return cuda_fail(plan, e, "leaf offset check");
         plan->launches += 1;
     }
     if (need_rho) {
@@ -503,8 +487,8 @@ q2x_status run_elements(q2x_plan_t plan, int kind, int dens, int64_t n_elem, int
             if (e != cudaSuccess) return cuda_fail(plan, e, "tile kernel occupancy query");
             if (tocc <= 0) return fail(plan, Q2X_ERR_CUDA, "tile kernel does not fit on the device (smem %zu)", f.smem);
         }
-        e = q2x::leaf_tiles_build(leaf_off, n_leaves, kLeafTileElems, tcombo, bin, w, plan->stream);
-        if (e == cudaSuccess) e = cudaMemsetAsync(w.counter, 0, sizeof(unsigned long long), plan->stream);
+        int built = 0;
+        e = q2x::leaf_tiles_build(leaf_off, n_leaves, kLeafTileElems, tcombo, bin, w, plan->d_err, &built, plan->stream);
         if (e != cudaSuccess) return cuda_fail(plan, e, "leaf tile list");
         q2x::BatchArgs b{};
         b.kind[kind].n_elem = n_elem;
@@ -544,7 +528,7 @@ q2x_status run_elements(q2x_plan_t plan, int kind, int dens, int64_t n_elem, int
         }
         e = q2x::leaf_tiles_combine(partial[0], w.slot_off, leaf_off, np, n_leaves, coef0, accumulate, plan->stream);
         if (e != cudaSuccess) return cuda_fail(plan, e, "leaf tile combine");
-        plan->launches += 5;
+        plan->launches += built + 2;
         return Q2X_OK;
     }
 
@@ -616,7 +600,7 @@ q2x_status q2x_galerkin_directions(q2x_plan_t plan, int64_t n_elem, int64_t n_ve
                                    const double* leaf_c, int layer, const double* w, double* out, bool* taken)
 {
     const int p = plan->p_max, np = (p + 1) * (p + 1);
-    const q2x::DirShape shape = q2x::dir_shape(p, 1, n_elem, n_leaves);
+    const q2x::DirShape shape = q2x::dir_shape(p, 1, n_elem, n_leaves, plan->num_sms);
     const size_t bytes = leaf_tile_ws_bytes(n_elem, n_leaves, np, shape.T, 0);
     *taken = n_leaves < ((int64_t)1 << 31) && bytes <= ((size_t)8 << 30);
     if (!*taken) return Q2X_OK;
@@ -629,8 +613,8 @@ q2x_status q2x_galerkin_directions(q2x_plan_t plan, int64_t n_elem, int64_t n_ve
     q2x::LeafTileWork lw;
     leaf_tile_carve(static_cast<unsigned char*>(plan->ws), n_elem, n_leaves, np, shape.T, 0, lw, nullptr);
     lw.max_slots = (int64_t)1 << 62;  // tiles keep no partial rows here: none is dropped for want of one
-    e = q2x::leaf_tiles_build(leaf_off, n_leaves, shape.T, 0, 0, lw, plan->stream);
-    if (e == cudaSuccess) e = cudaMemsetAsync(lw.counter, 0, sizeof(unsigned long long), plan->stream);
+    int built = 0;
+    e = q2x::leaf_tiles_build(leaf_off, n_leaves, shape.T, 0, 0, lw, nullptr, &built, plan->stream);
     if (e != cudaSuccess) return cuda_fail(plan, e, "leaf tile list");
     a.kind = q2x::BatchKind{n_elem, n_vert, vxyz, vxyz + n_vert, vxyz + 2 * n_vert, idx, sigma};
     a.n_leaves = n_leaves;
@@ -654,7 +638,7 @@ q2x_status q2x_galerkin_directions(q2x_plan_t plan, int64_t n_elem, int64_t n_ve
     const int64_t grid = std::min<int64_t>((int64_t)occ * plan->num_sms, lw.max_tiles);
     e = f.launch(a, shape.nt, shape.T, (int)grid, plan->stream);
     if (e != cudaSuccess) return cuda_fail(plan, e, "direction kernel launch");
-    plan->launches += 4;
+    plan->launches += built + 1;
     return Q2X_OK;
 }
 
@@ -799,7 +783,7 @@ q2x_status q2x_reserve(q2x_plan_t plan, int64_t n_elem, int64_t n_leaves)
     else
         for (int layers = 1; layers <= 3; ++layers)
             tile = std::max(tile, leaf_tile_ws_bytes(n_elem, n_leaves, np,
-                                                     q2x::dir_shape(plan->p_max, layers, n_elem, n_leaves).T, layers));
+                                                     q2x::dir_shape(plan->p_max, layers, n_elem, n_leaves, plan->num_sms).T, layers));
     if (tile > ((size_t)8 << 30)) tile = 0;  // such calls run the element kernel
     const size_t bytes = std::max(elem, tile) + align_up(sizeof(double) * (size_t)n_leaves, 256) +
                          align_up(sizeof(int) * (size_t)n_leaves, 256);
@@ -872,8 +856,8 @@ q2x_status q2x_leaf_reduce(q2x_plan_t plan, int64_t n_elem, int p, const double*
     cudaError_t e = cudaSetDevice(plan->device);
     if (e != cudaSuccess) return cuda_fail(plan, e, "cudaSetDevice");
     const int np = (p + 1) * (p + 1);
-    check_leaf_off_kernel<<<(unsigned)((n_leaves + 1 + 255) / 256), 256, 0, plan->stream>>>(leaf_off, n_leaves, n_elem,
-                                                                                           plan->d_err);
+    e = q2x::check_leaf_off(leaf_off, n_leaves, n_elem, plan->d_err, plan->stream);
+    if (e != cudaSuccess) return cuda_fail(plan, e, "leaf offset check");
     const int warps = 8;
     const int64_t units = n_leaves * (int64_t)np;  // (leaf, column) threads
     leaf_reduce_kernel<<<(unsigned)((units + warps * 32 - 1) / (warps * 32)), warps * 32, 0, plan->stream>>>(
@@ -931,8 +915,8 @@ q2x_status q2x_leaf_reduce_weighted(q2x_plan_t plan, int64_t n_elem, int p, cons
     if (n_leaves == 0) return Q2X_OK;
     cudaError_t e = cudaSetDevice(plan->device);
     if (e != cudaSuccess) return cuda_fail(plan, e, "cudaSetDevice");
-    check_leaf_off_kernel<<<(unsigned)((n_leaves + 1 + 255) / 256), 256, 0, plan->stream>>>(leaf_off, n_leaves, n_elem,
-                                                                                           plan->d_err);
+    e = q2x::check_leaf_off(leaf_off, n_leaves, n_elem, plan->d_err, plan->stream);
+    if (e != cudaSuccess) return cuda_fail(plan, e, "leaf offset check");
     const int warps = 8;
     const int64_t units = n_leaves * (int64_t)((np + 31) / 32);  // (leaf, 32-column group) warps
     const unsigned grid = (unsigned)((units + warps - 1) / warps);

@@ -230,9 +230,12 @@ constexpr int kLeafTileBlock = 1024;  // leaves per block of the tile count
 inline int64_t leaf_tile_blocks(int64_t n_leaves) { return (n_leaves + kLeafTileBlock - 1) / kLeafTileBlock; }
 inline int64_t leaf_tile_max_tiles(int64_t n_leaves, int64_t n_elem, int64_t T) { return n_leaves + (n_elem + T - 1) / T; }
 inline int64_t leaf_tile_max_slots(int64_t n_elem, int64_t T) { return 2 * ((n_elem + T - 1) / T); }
-// tile list of leaf_off with at most T elements per tile
+// leaf_off non-decreasing from 0 to n_elem, or Q2X_DEVERR_LEAF_OFF to *err
+cudaError_t check_leaf_off(const int64_t* leaf_off, int64_t n_leaves, int64_t n_elem, unsigned* err, cudaStream_t st);
+// tile list of leaf_off with at most T elements per tile, the offset check
+// (unless err is NULL) and the counter's reset; *launches: kernels launched
 cudaError_t leaf_tiles_build(const int64_t* leaf_off, int64_t n_leaves, int64_t T, int combo, int bin,
-                             const LeafTileWork& w, cudaStream_t st);
+                             const LeafTileWork& w, unsigned* err, int* launches, cudaStream_t st);
 // coef rows of the multi-tile leaves (sum of their partial rows in order) and,
 // unless accumulating, zero rows for empty leaves
 cudaError_t leaf_tiles_combine(const double* partial, const int64_t* slot_off, const int64_t* leaf_off,

@@ -64,7 +64,7 @@ const DirFns& dir_fns(int cls, int combo)
 // 3 a leaf 5.7 with 64, 8.9 with 256; p = 8: 13 a leaf 0.80 with 64, 1.55 with
 // 256; 53 a leaf 256 is ahead at p = 12, 1.12 against 1.18 ms, and 40 tetrahedra a
 // leaf at p = 10, 0.26 against 0.31, but behind at p = 8, 0.70 against 0.56).
-DirShape dir_shape(int p, int layers, int64_t n_elem, int64_t n_leaves)
+DirShape dir_shape(int p, int layers, int64_t n_elem, int64_t n_leaves, int num_sms)
 {
     const double mean = (double)n_elem / (double)std::max<int64_t>(n_leaves, 1);
     DirShape s{0, 256, 0};
@@ -77,6 +77,11 @@ DirShape dir_shape(int p, int layers, int64_t n_elem, int64_t n_leaves)
         s.cls = (p >= 12 && s.nt == 128) ? 0 : 1;
     }
     s.T = dir_tile_elems(p, s.nt);
+    // few elements: smaller tiles, down to one element a group, so that every
+    // SM has one (1,280 triangles in one leaf at p = 10: 58 us a call with 7
+    // full tiles, 39 with 56 tiles of one element a group)
+    const int64_t spread = n_elem / std::max(num_sms, 1);
+    if (spread < s.T) s.T = (int)std::max<int64_t>(std::min(s.T, s.nt / (p + 1)), spread);
     return s;
 }
 

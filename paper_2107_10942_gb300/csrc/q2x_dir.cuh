@@ -904,7 +904,7 @@ const DirFns& dir_fns(int cls, int combo);
 struct DirShape {
     int cls, nt, T;
 };
-DirShape dir_shape(int p, int layers, int64_t n_elem, int64_t n_leaves);
+DirShape dir_shape(int p, int layers, int64_t n_elem, int64_t n_leaves, int num_sms);
 // Elements a tile may hold: eight a group (the number format's head room), at
 // most one a thread (the frames).
 inline int dir_tile_elems(int p, int nt)

@@ -73,6 +73,19 @@ __device__ __forceinline__ void leaf_counts(const int64_t* leaf_off, int64_t L, 
     ns = nt >= 2 ? nt : 0;
 }
 
+// leaf_off must be non-decreasing with leaf_off[0] = 0, leaf_off[n_leaves] = n_elem
+__global__ void check_leaf_off_kernel(const int64_t* off, int64_t n_leaves, int64_t n_elem, unsigned* err)
+{
+    const int64_t L = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (L > n_leaves) return;
+    const int64_t o = off[L];
+    bool bad = (o < 0 || o > n_elem);
+    if (L == 0 && o != 0) bad = true;
+    if (L == n_leaves && o != n_elem) bad = true;
+    if (L < n_leaves && off[L + 1] < o) bad = true;
+    if (bad) atomicOr(err, Q2X_DEVERR_LEAF_OFF);
+}
+
 __global__ void __launch_bounds__(kLeafTileBlock) leaf_tile_count_kernel(const int64_t* leaf_off, int64_t n_leaves,
                                                                        int64_t T, LeafTileWork w)
 {
@@ -114,6 +127,28 @@ __global__ void __launch_bounds__(kLeafTileBlock) leaf_tile_scan_kernel(int64_t 
     if (threadIdx.x == 0) *w.n_tiles = carry[0] < w.max_tiles ? carry[0] : w.max_tiles;
 }
 
+// tile i of the nt tiles of leaf L (elements e0 .. e1, balanced sizes) to
+// entry `at` of the list; s0 the leaf's first partial row
+__device__ __forceinline__ void write_tile(const LeafTileWork& w, int64_t L, int64_t nt, int64_t i, int64_t at,
+                                           int64_t s0, int64_t e0, int64_t e1, int combo, int bin)
+{
+    const int64_t chunk = (e1 - e0 + nt - 1) / nt;
+    BatchTile t;
+    t.combo = combo;
+    t.bin = bin;
+    t.leaf = (int32_t)L;
+    t.flags = (nt == 1) ? 1 : 0;
+    t.slot = (nt == 1) ? 0 : s0 + i;
+    t.e_lo = e0 + i * chunk;
+    t.e_hi = (t.e_lo + chunk < e1) ? t.e_lo + chunk : e1;
+    if (nt > 1 && s0 + i >= w.max_slots) {  // no partial row left (bad offsets only): an empty tile
+        t.flags = 1;
+        t.slot = 0;
+        t.e_hi = t.e_lo;
+    }
+    w.tiles[at] = t;
+}
+
 // one thread per leaf: its tiles (balanced sizes, at most T elements) and
 // its partial-row offset
 __global__ void leaf_tile_fill_kernel(const int64_t* leaf_off, int64_t n_leaves, int64_t T, int combo, int bin,
@@ -132,23 +167,58 @@ __global__ void leaf_tile_fill_kernel(const int64_t* leaf_off, int64_t n_leaves,
     if (nt == 0) return;
     int64_t e0, e1;
     leaf_range(leaf_off, L, w.n_elem, e0, e1);
-    const int64_t chunk = (e1 - e0 + nt - 1) / nt;
     for (int64_t i = 0; i < nt; ++i) {
         if (t0 + i >= w.max_tiles) break;  // past the counted tiles (bad offsets only)
-        BatchTile t;
-        t.combo = combo;
-        t.bin = bin;
-        t.leaf = (int32_t)L;
-        t.flags = (nt == 1) ? 1 : 0;
-        t.slot = (nt == 1) ? 0 : s0 + i;
-        t.e_lo = e0 + i * chunk;
-        t.e_hi = (t.e_lo + chunk < e1) ? t.e_lo + chunk : e1;
-        if (nt > 1 && s0 + i >= smax) {  // no partial row left (bad offsets only): an empty tile
-            t.flags = 1;
-            t.slot = 0;
-            t.e_hi = t.e_lo;
+        write_tile(w, L, nt, i, t0 + i, s0, e0, e1, combo, bin);
+    }
+}
+
+// All of the above for at most kLeafTileBlock leaves, in one launch of one
+// block: the offset check, the counts and their scan, the tiles (over all
+// threads, each tile's leaf by bisection of the prefix sums) and the tile
+// counter's reset.  A small call's five launches took longer than its work.
+__global__ void __launch_bounds__(kLeafTileBlock) leaf_tile_small_kernel(const int64_t* leaf_off, int64_t n_leaves,
+                                                                       int64_t T, int combo, int bin, LeafTileWork w,
+                                                                       unsigned* err)
+{
+    __shared__ int64_t s_pre[kLeafTileBlock + 1], tot_t, tot_s;
+    const int64_t L = threadIdx.x;
+    int64_t nt = 0, ns = 0;
+    if (L < n_leaves) {
+        leaf_counts(leaf_off, L, T, w.n_elem, nt, ns);
+        const int64_t o0 = leaf_off[L], o1 = leaf_off[L + 1];
+        if (o0 < 0 || o0 > w.n_elem || o1 < o0 || o1 > w.n_elem || (L == 0 && o0 != 0) ||
+            (L == n_leaves - 1 && o1 != w.n_elem))
+            if (err) atomicOr(err, Q2X_DEVERR_LEAF_OFF);
+    }
+    int64_t et, es;
+    block_scan2(nt, ns, et, es, &tot_t, &tot_s);
+    __syncthreads();
+    s_pre[L] = et;
+    const int64_t smax = w.max_slots;
+    if (L < n_leaves) w.slot_off[L] = es < smax ? es : smax;
+    if (L == 0) {
+        s_pre[kLeafTileBlock] = tot_t;
+        w.slot_off[n_leaves] = tot_s < smax ? tot_s : smax;
+        *w.n_tiles = tot_t < w.max_tiles ? tot_t : w.max_tiles;
+        *w.counter = 0;
+    }
+    __syncthreads();
+    const int64_t n_tiles = tot_t < w.max_tiles ? tot_t : w.max_tiles;
+    for (int64_t i = threadIdx.x; i < n_tiles; i += kLeafTileBlock) {
+        int lo = 0, hi = kLeafTileBlock - 1;  // the last leaf whose first tile is at most i and that has tiles
+        while (lo < hi) {
+            const int mid = (lo + hi + 1) >> 1;
+            if (s_pre[mid] <= i)
+                lo = mid;
+            else
+                hi = mid - 1;
         }
-        w.tiles[t0 + i] = t;
+        // (leaves without tiles share their successor's prefix: lo is the last of them, the one with tiles)
+        int64_t e0, e1;
+        leaf_range(leaf_off, lo, w.n_elem, e0, e1);
+        const int64_t cnt = s_pre[lo + 1] - s_pre[lo], k = i - s_pre[lo];
+        write_tile(w, lo, cnt, k, i, w.slot_off[lo], e0, e1, combo, bin);
     }
 }
 
@@ -193,9 +263,28 @@ __global__ void leaf_tile_combine_kernel(const double* __restrict__ partial, con
 
 }  // namespace
 
-cudaError_t leaf_tiles_build(const int64_t* leaf_off, int64_t n_leaves, int64_t T, int combo, int bin,
-                             const LeafTileWork& w, cudaStream_t st)
+cudaError_t check_leaf_off(const int64_t* leaf_off, int64_t n_leaves, int64_t n_elem, unsigned* err, cudaStream_t st)
 {
+    check_leaf_off_kernel<<<(unsigned)((n_leaves + 1 + 255) / 256), 256, 0, st>>>(leaf_off, n_leaves, n_elem, err);
+    return cudaGetLastError();
+}
+
+cudaError_t leaf_tiles_build(const int64_t* leaf_off, int64_t n_leaves, int64_t T, int combo, int bin,
+                             const LeafTileWork& w, unsigned* err, int* launches, cudaStream_t st)
+{
+    if (n_leaves <= kLeafTileBlock) {
+        leaf_tile_small_kernel<<<1, kLeafTileBlock, 0, st>>>(leaf_off, n_leaves, T, combo, bin, w, err);
+        *launches = 1;
+        return cudaGetLastError();
+    }
+    *launches = 3;
+    if (err) {
+        const cudaError_t e = check_leaf_off(leaf_off, n_leaves, w.n_elem, err, st);
+        if (e != cudaSuccess) return e;
+        *launches = 4;
+    }
+    const cudaError_t e = cudaMemsetAsync(w.counter, 0, sizeof(unsigned long long), st);
+    if (e != cudaSuccess) return e;
     const int64_t nb = leaf_tile_blocks(n_leaves);
     leaf_tile_count_kernel<<<(unsigned)nb, kLeafTileBlock, 0, st>>>(leaf_off, n_leaves, T, w);
     leaf_tile_scan_kernel<<<1, kLeafTileBlock, 0, st>>>(nb, w);
