@@ -204,6 +204,23 @@ cudaError_t batch_group_launch(const BatchArgs& b, int64_t t0, int64_t t1, int g
 const BatchGroupFns* batch_group_table_f32();
 const BatchGroupFns* batch_group_table_f64();
 
+// sum of a column's partial rows s0 .. s1 - 1 in order, eight loads in flight
+__device__ __forceinline__ double sum_rows(const double* __restrict__ col, int64_t s0, int64_t s1, int np,
+                                           int accumulate, double old)
+{
+    double acc = 0.0;
+    int64_t s = s0;
+    for (; s + 8 <= s1; s += 8) {
+        double v[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) v[u] = col[(s + u) * np];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) acc += v[u];
+    }
+    for (; s < s1; ++s) acc += col[s * np];
+    return accumulate ? old + acc : acc;
+}
+
 // coef[L] (+)= sum of the partial rows slot_off[L] .. slot_off[L+1]-1, in order
 __global__ void q2x_batch_combine(const double* __restrict__ partial, const int64_t* __restrict__ slot_off,
                                   int np, int64_t n_leaves, double* coef, int accumulate);

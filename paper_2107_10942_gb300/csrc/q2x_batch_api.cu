@@ -16,16 +16,13 @@ namespace q2x {
 __global__ void q2x_batch_combine(const double* __restrict__ partial, const int64_t* __restrict__ slot_off,
                                   int np, int64_t n_leaves, double* coef, int accumulate)
 {
-    const int lane = threadIdx.x & 31;
-    const int64_t L = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    if (L >= n_leaves) return;
-    const int64_t s0 = slot_off[L], s1 = slot_off[L + 1];
-    for (int c = lane; c < np; c += 32) {
-        double acc = 0.0;
-        for (int64_t s = s0; s < s1; ++s) acc += partial[s * np + c];
-        double* d = coef + L * np + c;
-        *d = accumulate ? *d + acc : acc;
-    }
+    // one warp per (leaf, 32 columns): a chain of loads each, so many of them
+    const int chunks = (np + 31) >> 5;
+    const int64_t warp = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), L = warp / chunks;
+    const int c = (int)(warp % chunks) * 32 + (threadIdx.x & 31);
+    if (L >= n_leaves || c >= np) return;
+    double* d = coef + L * np + c;
+    *d = sum_rows(partial + c, slot_off[L], slot_off[L + 1], np, accumulate, accumulate ? *d : 0.0);
 }
 }  // namespace q2x
 
@@ -256,8 +253,8 @@ q2x_status build_batch(q2x_plan_t plan, const q2x_batch_desc* d, int tile_elems,
         for (int i = 0; i < nbr && e == cudaSuccess; ++i) e = cudaStreamWaitEvent(cs, ev_join[i], 0);
     }
     if (e == cudaSuccess) {
-        const int warps = 8;
-        q2x::q2x_batch_combine<<<(unsigned)((nl + warps - 1) / warps), warps * 32, 0, cs>>>(
+        const int64_t warps = 8, n_warps = nl * ((np + 31) / 32);
+        q2x::q2x_batch_combine<<<(unsigned)((n_warps + warps - 1) / warps), warps * 32, 0, cs>>>(
             b->d_partial, b->d_slot_off, np, nl, b->coef, b->accumulate);
         e = cudaGetLastError();
     }

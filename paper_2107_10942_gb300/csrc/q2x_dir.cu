@@ -78,8 +78,8 @@ DirShape dir_shape(int p, int layers, int64_t n_elem, int64_t n_leaves, int num_
     }
     s.T = dir_tile_elems(p, s.nt);
     // few elements: smaller tiles, down to one element a group, so that every
-    // SM has one (1,280 triangles in one leaf at p = 10: 58 us a call with 7
-    // full tiles, 39 with 56 tiles of one element a group)
+    // SM has one (1,280 triangles in one leaf at p = 10: 56 tiles of one element
+    // a group take 19 us less than 7 full tiles)
     const int64_t spread = n_elem / std::max(num_sms, 1);
     if (spread < s.T) s.T = (int)std::max<int64_t>(std::min(s.T, s.nt / (p + 1)), spread);
     return s;

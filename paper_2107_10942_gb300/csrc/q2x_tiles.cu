@@ -3,6 +3,7 @@
 // tile kernel (see q2x_batch.cuh), and its combine.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cstdint>
 
 #include "q2x_batch.cuh"
@@ -222,21 +223,25 @@ __global__ void __launch_bounds__(kLeafTileBlock) leaf_tile_small_kernel(const i
     }
 }
 
-// one warp per 32 leaves: each lane reads one leaf's slot and element
-// ranges; the warp then handles, one after the other, the leaves that have
-// work (several tiles: their partial rows summed in slot order; empty and
-// not accumulating: a zero row), columns over the lanes
+// One warp per (lpw leaves, every chunks-th 32 columns): each lane reads one leaf's slot and
+// element ranges; the warp then handles, one after the other, the leaves that
+// have work (several tiles: their partial rows summed in slot order; empty and
+// not accumulating: a zero row).  It is a chain of loads, so the warps are as
+// many as the chip holds (leaf_tiles_combine), and never fewer leaves than
+// give that.
 __global__ void leaf_tile_combine_kernel(const double* __restrict__ partial, const int64_t* __restrict__ slot_off,
                                          const int64_t* __restrict__ leaf_off, int np, int64_t n_leaves, double* coef,
-                                         int accumulate)
+                                         int accumulate, int lpw, int chunks)
 {
     const int lane = threadIdx.x & 31;
-    const int64_t L0 = ((int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * 32;
+    const int64_t warp = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+    const int64_t L0 = warp / chunks * lpw;
     if (L0 >= n_leaves) return;  // warp-uniform
     const int64_t L = L0 + lane;
+    const int c0 = (int)(warp % chunks) * 32 + lane;
     long long s0 = 0, s1 = 0;
     bool work = false;
-    if (L < n_leaves) {
+    if (lane < lpw && L < n_leaves) {
         s0 = slot_off[L];
         s1 = slot_off[L + 1];
         const bool empty = __ldg(leaf_off + L + 1) == __ldg(leaf_off + L);
@@ -248,15 +253,9 @@ __global__ void leaf_tile_combine_kernel(const double* __restrict__ partial, con
         const int r = __ffs(mask) - 1;
         mask &= mask - 1;
         const long long a0 = __shfl_sync(0xffffffffu, s0, r), a1 = __shfl_sync(0xffffffffu, s1, r);
-        double* row = coef + (L0 + r) * np;
-        if (a1 == a0) {  // an empty leaf is zero
-            for (int c = lane; c < np; c += 32) row[c] = 0.0;
-        } else {
-            for (int c = lane; c < np; c += 32) {
-                double acc = 0.0;
-                for (long long sl = a0; sl < a1; ++sl) acc += partial[sl * np + c];
-                row[c] = accumulate ? row[c] + acc : acc;
-            }
+        for (int c = c0; c < np; c += 32 * chunks) {
+            double* at = coef + (L0 + r) * np + c;
+            *at = a1 == a0 ? 0.0 : sum_rows(partial + c, a0, a1, np, accumulate, accumulate ? *at : 0.0);
         }
     }
 }
@@ -295,10 +294,19 @@ cudaError_t leaf_tiles_build(const int64_t* leaf_off, int64_t n_leaves, int64_t 
 cudaError_t leaf_tiles_combine(const double* partial, const int64_t* slot_off, const int64_t* leaf_off, int np,
                                int64_t n_leaves, double* coef, int accumulate, cudaStream_t st)
 {
+    // as many warps as 152 SMs hold (64 each), then more leaves and columns a
+    // warp.  Whole calls at p = 10, 32 leaves and all columns a warp -> so:
+    // 1 leaf of 56 tiles 42.0 -> 27.6 us, some 50 leaves of 0.8 k triangles
+    // 249 -> 113, 3 k of 0.2 k 1218 -> 1133 (FP32-mixed 309 -> 225), 12 k
+    // (FP32-mixed) 892 -> 761; at 240 k leaves both are the same
     const int warps = 8;
-    const int64_t n_warps = (n_leaves + 31) / 32;
+    const int64_t cap = 152 * 64, groups = (n_leaves + 31) / 32;
+    const int chunks = (int)std::min<int64_t>((np + 31) / 32, std::max<int64_t>(1, cap / groups));
+    int lpw = 1;
+    while (lpw < 32 && n_leaves * chunks > cap * lpw) lpw *= 2;
+    const int64_t n_warps = (n_leaves + lpw - 1) / lpw * chunks;
     leaf_tile_combine_kernel<<<(unsigned)((n_warps + warps - 1) / warps), warps * 32, 0, st>>>(
-        partial, slot_off, leaf_off, np, n_leaves, coef, accumulate);
+        partial, slot_off, leaf_off, np, n_leaves, coef, accumulate, lpw, chunks);
     return cudaGetLastError();
 }
 

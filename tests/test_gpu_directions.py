@@ -149,9 +149,10 @@ def test_accumulate_and_repeat(q2x):
 
 
 @pytest.mark.parametrize("precision", ["fp64", "fp32"])
-@pytest.mark.parametrize("n_leaves,p", [(1, 3), (3, 20), (1023, 9), (1024, 3), (1025, 3), (12000, 9)])
+@pytest.mark.parametrize("n_leaves,p", [(1, 3), (3, 20), (1023, 9), (1024, 3), (1025, 3), (12000, 9), (100000, 9)])
 def test_tile_list_and_offset_check(q2x, n_leaves, p, precision):
-    """The tile list's one-block build and the general one about their border:
+    """The tile list's one-block build and the general one about their border,
+    and the combine with one to 32 leaves and all or fewer columns a warp:
     empty leaves at both ends, some of many tiles, the same sums as the
     per-element rows, and bad offsets reported."""
     rng = np.random.default_rng(n_leaves)
