@@ -323,6 +323,24 @@ q2x_status q2x_translate_rt(q2x_plan_t plan, int p, int64_t n_src, const double*
                             const double* rt, const int32_t* t_idx, int64_t n_dst, const int64_t* dst_off,
                             double* dst_coef, int accumulate);
 
+/* Table for q2x_translate_octants: shifts (+-h, +-h, +-h), degree p, norm as
+ * the plan's (0 COEFF, 1 MOMENT), about n_dst destinations.  Host code, no
+ * GPU: with table NULL the bytes it needs, else it is written to table (host,
+ * `bytes` long, 16-byte aligned) and the bytes used are returned; -1 for bad
+ * arguments.  The caller copies it to the device. */
+int64_t q2x_octant_table(int p, int norm, double h, int64_t n_dst, void* table, int64_t bytes);
+
+/* q2x_translate for one level of an octree, children to parents: source s
+ * lies in octant oct[s] of its destination (int32, device; bits 0, 1, 2 set
+ * where x, y, z of src centre - dst centre are -h, else +h).  table (device)
+ * is the one for this p, norm, h and n_dst; another p, norm or split sets
+ * bit 1 of the device error word and writes nothing.  An octant outside 0..7
+ * sets bit 1 and that source adds zero.  Sources of one destination are
+ * combined before they are translated: one translation a destination. */
+q2x_status q2x_translate_octants(q2x_plan_t plan, int p, int64_t n_src, const double* src_coef, const void* table,
+                                 const int32_t* oct, int64_t n_dst, const int64_t* dst_off, double* dst_coef,
+                                 int accumulate);
+
 /* Far-field evaluation (the M2P step fed by the leaf or box coefficients):
  * out[t] (+)= sum over the expansions e listed for target t of
  *   phi_e(x_t) = sum_{n<=p} sum_{|m|<=n} F_n^m S_n^m(x_t - c_e)      (Eq. (bas3))

@@ -37,6 +37,7 @@ _SIGNATURES = {
     "q2x_translate": [_p, _i, _i64, _p, _p, _i64, _p, _p, _p, _i],
     "q2x_translation_rows": [_p, _i, _i64, _p, _p],
     "q2x_translate_rt": [_p, _i, _i64, _p, _i64, _p, _p, _i64, _p, _p, _i],
+    "q2x_translate_octants": [_p, _i, _i64, _p, _p, _p, _i64, _p, _p, _i],
     "q2x_evaluate": [_p, _i, _i64, _p, _p, _i64, _p, _p, _p, _p, _i],
     "q2x_evaluate_curl": [_p, _i, _i64, _p, _p, _i64, _p, _p, _p, _p, _i],
     "q2x_segments_vector": [_p, _i64, _i64, _p, _p, _p, _i64, _p, _p, _p, _p, _p, _i],
@@ -92,6 +93,8 @@ def lib():
             L.q2x_workspace_bytes.restype = _c.c_int64
             L.q2x_launch_count.argtypes = [_p]
             L.q2x_launch_count.restype = _c.c_int64
+            L.q2x_octant_table.argtypes = [_i, _i, _c.c_double, _i64, _p, _i64]
+            L.q2x_octant_table.restype = _c.c_int64
             _LIB = L
     return _LIB
 

@@ -41,6 +41,25 @@ def _need(t, dtype, name, shape=None):
     return t
 
 
+def octant_table_host(p, norm, h, n_dst):
+    """The table of q2x_octant_table as a uint8 host tensor."""
+    n = lib().q2x_octant_table(p, norm, float(h), n_dst, None, 0)
+    if n < 0:
+        raise ValueError("octant table: bad arguments")
+    buf = torch.empty(n, dtype=torch.uint8)
+    if lib().q2x_octant_table(p, norm, float(h), n_dst, _ptr(buf), n) != n:
+        raise ValueError("octant table: bad arguments")
+    return buf
+
+
+class OctantTable:
+    """Plan.octant_table: the device table and what it was made for."""
+
+    def __init__(self, p, norm, n_dst, data):
+        self.p, self.norm, self.n_dst = p, norm, n_dst
+        self.data = _need(data, torch.uint8, "table")
+
+
 class PlanGraph:
     """A captured sequence of q2x calls (Plan.capture)."""
 
@@ -303,6 +322,36 @@ class Plan:
                                      _ptr(dst_off), _ptr(dst_coef), int(bool(accumulate))), self._h)
         return dst_coef
 
+
+    def octant_table(self, h, n_dst, p=None, device="cuda"):
+        """Device table of translate_octants for shifts (+-h, +-h, +-h) and
+        n_dst destinations (q2x_octant_table)."""
+        p = self.p_max if p is None else int(p)
+        return OctantTable(p, self.norm, int(n_dst), octant_table_host(p, self.norm, h, n_dst).to(device))
+
+    def translate_octants(self, src_coef, table, octant, dst_off, dst_coef=None, accumulate=False, p=None):
+        """translate() for one octree level, children to parents: source s lies
+        in octant[s] (bits 0, 1, 2: x, y, z of its shift negative) of its
+        destination (q2x_translate_octants)."""
+        p = self.p_max if p is None else int(p)
+        nc = n_coef(p)
+        _need(src_coef, torch.float64, "src_coef")
+        if src_coef.dim() != 2 or src_coef.shape[1] != nc:
+            raise ValueError("src_coef must be (n_src, (p+1)^2)")
+        n_src = src_coef.shape[0]
+        _need(octant, torch.int32, "octant", (n_src,))
+        _need(dst_off, torch.int64, "dst_off")
+        n_dst = dst_off.shape[0] - 1
+        if dst_coef is None:
+            if accumulate:
+                raise ValueError("accumulate=True needs an output tensor")
+            dst_coef = torch.empty((n_dst, nc), dtype=torch.float64, device=src_coef.device)
+        _need(dst_coef, torch.float64, "dst_coef", (n_dst, nc))
+        if (table.p, table.norm, table.n_dst) != (p, self.norm, n_dst):
+            raise ValueError("table is not the one of this p, norm and number of destinations")
+        check(lib().q2x_translate_octants(self._h, p, n_src, _ptr(src_coef), _ptr(table.data), _ptr(octant), n_dst,
+                                          _ptr(dst_off), _ptr(dst_coef), int(bool(accumulate))), self._h)
+        return dst_coef
 
     def evaluate(self, coef, exp_c, tgt, tgt_off=None, exp_idx=None, out=None, accumulate=False, p=None):
         """Far-field potential at the targets tgt (3, n_tgt) of the expansions
