@@ -204,6 +204,14 @@ cudaError_t batch_group_launch(const BatchArgs& b, int64_t t0, int64_t t1, int g
 const BatchGroupFns* batch_group_table_f32();
 const BatchGroupFns* batch_group_table_f64();
 
+// offset L, 0 <= L <= n_leaves, out of [0, n_elem], above its successor, or not
+// 0 first and n_elem last
+__device__ __forceinline__ bool leaf_off_bad(const int64_t* off, int64_t L, int64_t n_leaves, int64_t n_elem)
+{
+    const int64_t o = off[L];
+    return o < 0 || o > n_elem || (L == 0 && o != 0) || (L == n_leaves ? o != n_elem : off[L + 1] < o);
+}
+
 // sum of a column's partial rows s0 .. s1 - 1 in order, eight loads in flight
 __device__ __forceinline__ double sum_rows(const double* __restrict__ col, int64_t s0, int64_t s1, int np,
                                            int accumulate, double old)

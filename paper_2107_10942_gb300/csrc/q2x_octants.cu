@@ -21,9 +21,9 @@
 // run of equal length a thread, entries in a transposed list, so no lane
 // waits; a run's share of an entry goes to a slot in shared memory, and one
 // thread an entry adds its slots in order (deterministic).
-// Measured at p = 12: 3,592 children of 916 parents 129 -> 29 us (FP64 pipe
-// 73 % busy), the levels above (229, 56, 8 and 1 parents) 55 + 20 + 19 + 17 ->
-// 12 + 9 + 9 + 9 us, latency of loads by then; the whole pass 214 -> 69 us.
+// Measured at p = 12: 3,592 children of 916 parents 129 -> 31 us (FP64 pipe
+// 73 % busy), the levels above (229, 56, 8 and 1 parents) 55 + 20 + 18 + 17 ->
+// 15 + 11 + 10 + 9 us, latency of loads by then; the whole pass 214 -> 69 us.
 // Errors against 128-bit sums are the general path's or smaller (degrees
 // weighted alike: 2.3e-16 against 3.4e-16 a level, 2.2e-15 and 2.0e-15 at the
 // root).

@@ -78,13 +78,7 @@ __device__ __forceinline__ void leaf_counts(const int64_t* leaf_off, int64_t L, 
 __global__ void check_leaf_off_kernel(const int64_t* off, int64_t n_leaves, int64_t n_elem, unsigned* err)
 {
     const int64_t L = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (L > n_leaves) return;
-    const int64_t o = off[L];
-    bool bad = (o < 0 || o > n_elem);
-    if (L == 0 && o != 0) bad = true;
-    if (L == n_leaves && o != n_elem) bad = true;
-    if (L < n_leaves && off[L + 1] < o) bad = true;
-    if (bad) atomicOr(err, Q2X_DEVERR_LEAF_OFF);
+    if (L <= n_leaves && leaf_off_bad(off, L, n_leaves, n_elem)) atomicOr(err, Q2X_DEVERR_LEAF_OFF);
 }
 
 __global__ void __launch_bounds__(kLeafTileBlock) leaf_tile_count_kernel(const int64_t* leaf_off, int64_t n_leaves,
