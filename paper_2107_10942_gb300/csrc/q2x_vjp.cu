@@ -15,7 +15,10 @@ cudaError_t launch_vjp(const q2x::VjpArgs& a, cudaStream_t st)
 {
     const int threads = 128;
     const unsigned grid = (unsigned)((a.n_elem + threads - 1) / threads);
-    q2x::q2x_tri_vjp_kernel<T, P><<<grid, threads, 0, st>>>(a);
+    if constexpr (sizeof(T) == 4)
+        q2x::q2x_tri_vjp_f32_kernel<P><<<grid, threads, 0, st>>>(a);
+    else
+        q2x::q2x_tri_vjp_kernel<T, P><<<grid, threads, 0, st>>>(a);
     return cudaGetLastError();
 }
 
