@@ -80,17 +80,27 @@ __device__ __forceinline__ V3 scale(V3 a, double s) { return V3{a.x * s, a.y * s
 // piece; D is formed as d02 / (R - s) where R + s would cancel.  The quotient
 // and the logarithm are one integer function of the five factors, and signs
 // are read from the bits: comparisons too would occupy the FP64 pipe.
-__device__ __forceinline__ double line_log(double sm, double sp, double Rm, double Rp, double d02, double L,
-                                           const NfTables& tab)
+// The value is log1p(L b c / (Sg e)).
+__device__ __forceinline__ void line_factors(double sm, double sp, double Rm, double Rp, double d02, double Sg,
+                                             double& b, double& c, double& e)
 {
-    const double Sg = Rm + Rp, sg = sm + sp;
+    const double sg = sm + sp;
     const bool behind = (nf_bits(sg) >> 63) != 0;
     const double a = behind ? Rp : Rm;
     const nf_u64 s = behind ? nf_bits(sp) ^ (1ull << 63) : nf_bits(sm);
     const bool ahead = (s >> 63) == 0;
     const double w = a + nf_double(s & 0x7fffffffffffffffull);
-    return nf_log1p_ratio(L, Sg + nf_double(nf_bits(sg) & 0x7fffffffffffffffull), ahead ? 1.0 : w, Sg,
-                          ahead ? w : d02, tab);
+    b = Sg + nf_double(nf_bits(sg) & 0x7fffffffffffffffull);
+    c = ahead ? 1.0 : w;
+    e = ahead ? w : d02;
+}
+__device__ __forceinline__ double line_log(double sm, double sp, double Rm, double Rp, double d02, double L,
+                                           const NfTables& tab)
+{
+    const double Sg = Rm + Rp;
+    double b, c, e;
+    line_factors(sm, sp, Rm, Rp, d02, Sg, b, c, e);
+    return nf_log1p_ratio(L, b, c, Sg, e, tab);
 }
 
 // A flat face in its own frame: origin x1, in-plane axes u (along the first
@@ -225,12 +235,30 @@ __device__ __forceinline__ void face_potential(const Face* __restrict__ Fp, V3 r
         const double Rv[4] = {R1, R2, R3, R1};
 #pragma unroll
         for (int i = 0; i < 3; ++i) {
-            // the edge's ends along it, and offset . m_i, m_i = (l_y, -l_x) the outward normal
-            const double sm = i ? px[i] * lx[i] + py[i] * ly[i] : -rx;
-            const double sp = i ? sm + Ls[i] : bx;
+            // offset . m_i, m_i = (l_y, -l_x) the outward normal
             const double t = i ? px[i] * ly[i] - py[i] * lx[i] : ry;
-            if ((nf_bits(t) & 0x7fffffffffffffffull) > tol && nf_bits(Ls[i]) != 0)  // else on the edge's line
-                S += t * line_log(sm, sp, Rv[i], Rv[i + 1], fma(t, t, h2), Ls[i], tab);
+            if ((nf_bits(t) & 0x7fffffffffffffffull) <= tol || nf_bits(Ls[i]) == 0) continue;  // on the edge's line
+            // From R+^2 - R-^2 = s+^2 - s-^2 the ratio is also (Sg + L) / (Sg - L),
+            // Sg = R- + R+: log1p(2 L / (Sg - L)), without the ends s-, s+ and d02
+            // (five to eight FP64 instructions fewer).  Taken from Sg of about
+            // 1.5 L on (0.585 in the exponent and leading bits): there the
+            // difference's rounding, 2x / ((x^2 - 1) log((x + 1) / (x - 1))) = 1.5
+            // times that of Sg at x = Sg / L, is no larger than the error of
+            // line_log's quotient; nearer the edge it grows without bound.
+            // 39.5 M pairs in leaves of 91 triangles: 6.68 -> 5.82 ms, in leaves of
+            // 5 times as many (fewer warps with a near edge) 5.66 -> 4.55 ms.
+            const double Sg = Rv[i] + Rv[i + 1];
+            double b = 2.0, c = 1.0, e = 1.0, d;
+            if ((int)(nf_bits(Sg) >> 32) - (int)(nf_bits(Ls[i]) >> 32) >= 613000) {
+                d = Sg - Ls[i];
+            } else {
+                // the edge's ends along it
+                const double sm = i ? px[i] * lx[i] + py[i] * ly[i] : -rx;
+                const double sp = i ? sm + Ls[i] : bx;
+                line_factors(sm, sp, Rv[i], Rv[i + 1], fma(t, t, h2), Sg, b, c, e);
+                d = Sg;
+            }
+            S += t * nf_log1p_ratio(Ls[i], b, c, d, e, tab);
         }
     }
     if (!in_plane) {
