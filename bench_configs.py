@@ -25,9 +25,17 @@ import workloads as W
 from bench import METRIC, UNIT, ClockSampler, L2_FLUSH_BYTES
 
 LINES = []
-# filled by run(): measured FP64 / FP32 FMA peaks (flop/s) of this device
+# filled by run(): measured FP64 / FP32 FMA peaks (flop/s) and the integer
+# multiply-add peak (32 x 32 + 64 bits, 1/s) of this device
 PEAKS = {}
 PEAK_SOURCE = "measured in this run (q2x_alu_peak_probe, FMA chains on every SM, CUDA events)"
+
+
+def _integer_roofline(madds, ms):
+    """Roofline entry of a kernel on 62-bit fixed point: its 32 x 32 + 64-bit
+    multiply-adds against their measured rate."""
+    return {"bound": "integer multiply-add", "achieved": madds / (ms * 1e-3) / 1e12, "peak": PEAKS["imad"] / 1e12,
+            "unit": "Tmadd/s", "frac": madds / (ms * 1e-3) / PEAKS["imad"]}
 
 
 def _norm_err(test, ref, rho, p, layer=0):
@@ -195,7 +203,7 @@ def run_icosphere_l3(args, dev):
     coef = torch.empty((1, (p + 1) ** 2), dtype=torch.float64, device=dev)
     fn = lambda: plan.triangles(d["vxyz"], d["idx"], d["sigma"], d["leaf_off"], d["leaf_c"], d["leaf_rho"], None,
                                 coef_single=coef)
-    # the step (check, element kernel, fix-up) as one CUDA graph, so that host
+    # the step (check and tile list, kernel, combine) as one CUDA graph, so that host
     # launch gaps do not enter the device time of this small problem
     g = plan.capture(fn)
     ms = _time(g.replay, args.steps, args.warmup, flush, stream)
@@ -220,25 +228,18 @@ def run_icosphere_l3(args, dev):
            "warmup": args.warmup, "ms_per_step": ms, "higher_is_better": True, "dtype": "f64", "data": "synthetic",
            "config": {"workload": "icosphere-L3: %d triangles, one expansion about the origin, p=10, single layer, "
                                   "constant density" % n_elem,
-                      "step": "one CUDA-graph replay (check, element kernel, fix-up)", "kernel_ms": kms / max(kn, 1),
-                      "note": "latency-bound: 40 warps of 32 triangles, one per SM sub-partition; each runs its "
-                              "round's FP64 chain alone on its sub-partition's FP64 pipe (about 2,000 FP64 "
-                              "instructions of 64 pipe cycles each), so the kernel cannot take less than about "
-                              "0.06 ms however many SMs are idle"},
+                      "step": "one CUDA-graph replay (offset check and tile list, direction kernel, combine)", "kernel_ms": kms / max(kn, 1),
+                      "note": "latency-bound: three launches, 56 tiles of one element a group"},
            "errors_vs_oracle": {"fp64": _norm_err(got, ref, prob["leaf_rho"], p)},
            "cpu_baseline": {"value": per_step / dt, "unit": UNIT, "kind": "oracle", "cores": orc.max_threads(),
                             "sample": "the whole workload, %d repetitions" % reps}})
 
 
-def translate_macs(p):
-    """complex multiply-adds of one translation of degree p (COEFF formula)"""
-    t = 0
-    for n in range(p + 1):
-        for m in range(n + 1):
-            for k in range(n + 1):
-                nn = n - k
-                t += max(0, min(k, nn - m) - max(-k, -nn - m) + 1)
-    return t
+def octant_terms(p):
+    """Multiply-adds of one parent's translation (the terms of its table)."""
+    from paper_2107_10942_gb300.q2x import octant_table_host
+    head = octant_table_host(p, 0, 1.0, 1 << 20)[:56].view(torch.int32)  # one chunk: its term count is word 8
+    return int(head[8])
 
 
 def run_upward(args, dev):
@@ -254,14 +255,14 @@ def run_upward(args, dev):
     up = Upward(plan, d["leaf_c"], -1.125, 2.25, depth)
     flush = torch.empty(L2_FLUSH_BYTES // 4, dtype=torch.float32, device=dev)
     stream = torch.cuda.current_stream()
-    # the pass as one CUDA graph (five levels, ten kernels, one host launch)
+    # the pass as one CUDA graph (five levels, five kernels, one host launch)
     up.capture(leaf)
     ms = _time(up.replay, args.steps, args.warmup, flush, stream)
     outs = up.replay()
     root = outs[-1].cpu().numpy()
     plan.sync()
     n_tr = sum(int(lv["dst_off"][-1]) for lv in up.levels)
-    flops = 8.0 * translate_macs(p) * n_tr
+    flops = 2.0 * octant_terms(p) * sum(lv["c"].shape[1] for lv in up.levels)
     # the root against quadrature of the whole sphere about the cube centre
     t0 = time.perf_counter()
     ref = orc.moments("triangle", prob["vxyz"], prob["idx"], prob["sigma"], p,
@@ -276,22 +277,19 @@ def run_upward(args, dev):
                                   "5 levels, one CUDA graph replay), p=12, FP64" % (prob["leaf_c"].shape[1], n_tr)},
            "roofline": {"bound": "alu", "achieved": flops / (ms * 1e-3) / 1e12, "peak": PEAKS["fp64"] / 1e12,
                         "unit": "TFLOP/s", "frac": flops / (ms * 1e-3) / PEAKS["fp64"],
-                        "flops_per_translation": 8 * translate_macs(p)},
+                        "flops_per_parent": 2 * octant_terms(p),
+                        "note": "multiply-adds of the parents' translations; the additions that combine the "
+                                "children first, at most 24 (p+1)^2 a parent, are not counted"},
            "errors_vs_oracle": {"root_vs_quadrature": err},
            "cpu_baseline": {"value": None, "note": "oracle quadrature of the root expansion over all %d triangles: "
                             "%.2f s" % (prob["idx"].shape[1], dt), "kind": "oracle", "cores": orc.max_threads()}})
 
 
-# FP64 flops per evaluation ncu counted as executed at p = 12:
-# (2 x 104.19 + 13.57 + 137.94) per elapsed cycle x 2.858 M cycles / 1,048,576
-EVAL_EXECUTED_FLOPS = (2 * 104.187417 + 13.573713 + 137.938271) * 2858268.0 / 1048576
-
-
-def eval_flops(p):
-    """Flops of one far-field evaluation (q2x_evaluate): per (n, m >= 0)
-    term a three-term step (3 multiplies, 1 FMA) and two FMAs = 9 flops; per
-    order m the update of T_m^m and the column's complex product (about 16)."""
-    return 9 * (p + 1) * (p + 2) // 2 + 16 * (p + 1)
+def eval_madds(p):
+    """Integer multiply-adds of one far-field evaluation (q2x_evaluate by
+    directions): per direction (p + 1) the dot product with the offset (18) and
+    per degree a complex product of 62-bit numbers (12)."""
+    return (p + 1) * (18 + 12 * p)
 
 
 def run_farfield(args, dev):
@@ -322,25 +320,18 @@ def run_farfield(args, dev):
     pick = rng.choice(n_tgt, 64, replace=False)
     ref = orc.farfield(rc, np.zeros(3), tg[:, pick].T, p)[0]
     err = float(np.max(np.abs(got[pick] - ref)) / np.max(np.abs(ref)))
-    flops = float(eval_flops(p)) * n_tgt
     _emit({"metric": "far-field evaluations/s (one p=12 expansion per target)", "value": n_tgt / (ms * 1e-3),
            "unit": "evaluations/s", "n_gpus": 1, "steps": args.steps, "warmup": args.warmup, "ms_per_step": ms,
            "higher_is_better": True, "dtype": "f64", "data": "synthetic",
            "config": {"workload": "root expansion of the level-7 sphere (p=12, from Q2X + upward pass) at %d targets "
                                   "on the radius-3 sphere" % n_tgt},
-           "roofline": {"bound": "alu", "achieved": flops / (ms * 1e-3) / 1e12, "peak": PEAKS["fp64"] / 1e12,
-                        "unit": "TFLOP/s", "frac": flops / (ms * 1e-3) / PEAKS["fp64"],
-                        "flops_per_evaluation": eval_flops(p),
-                        "executed": {"flops_per_evaluation": EVAL_EXECUTED_FLOPS,
-                                     "frac": EVAL_EXECUTED_FLOPS * n_tgt / (ms * 1e-3) / PEAKS["fp64"],
-                                     "source": "ncu DFMA/DADD/DMUL counts of one capture of this "
-                                               "kernel on this workload"}},
+           "roofline": dict(_integer_roofline(float(eval_madds(p)) * n_tgt, ms), madds_per_evaluation=eval_madds(p)),
            "errors_vs_oracle": {"series": err, "sampled_targets": 64}})
 
 
 def run_galerkin(args, dev):
     import paper_2107_10942_gb300 as q
-    from paper_2107_10942_gb300.roofline import element_flops
+    from paper_2107_10942_gb300.roofline import direction_madds
     import oracle as orc
     p, depth = 12, 5
     prob = W.cfg_sphere_linear(level=7, depth=depth, p=p)
@@ -367,20 +358,20 @@ def run_galerkin(args, dev):
     wn = w.cpu().numpy()
     ref = np.sum(P * wn[leaf_of[el]], axis=1)
     err = float(np.max(np.abs(got[el] - ref) / np.sum(np.abs(P * wn[leaf_of[el]]), axis=1)))
-    flops = (element_flops("triangle", "const", ("single",), p, point="order") + (p + 1) ** 2) * n_elem
+    # the element's recurrences, and one complex dot product a direction and degree
+    madds = (direction_madds("triangle", "const", ("single",), p) + 6 * (p + 1) ** 2) * n_elem
     _emit({"metric": "Galerkin element integrals/s (local expansion over each receiving triangle)",
            "value": n_elem / (ms * 1e-3), "unit": "elements/s", "n_gpus": 1, "steps": args.steps,
            "warmup": args.warmup, "ms_per_step": ms, "higher_is_better": True, "dtype": "f64", "data": "synthetic",
            "config": {"workload": "the level-7 sphere's %d triangles against random local expansions of its %d "
                                   "depth-5 leaves, p=12, single layer" % (n_elem, nl)},
-           "roofline": {"bound": "alu", "achieved": flops / (ms * 1e-3) / 1e12, "peak": PEAKS["fp64"] / 1e12,
-                        "unit": "TFLOP/s", "frac": flops / (ms * 1e-3) / PEAKS["fp64"]},
+           "roofline": _integer_roofline(madds, ms),
            "errors_vs_oracle": {"relative_to_sum_of_terms": err, "sampled_elements": 200}})
 
 
 def run_biot_savart(args, dev):
     import paper_2107_10942_gb300 as q
-    from paper_2107_10942_gb300.roofline import level_flops, point_level_order_flops
+    from paper_2107_10942_gb300.roofline import direction_madds
     from paper_2107_10942_gb300.upward import Upward
     p = 12
     m = W.cfg_mixed_ball()
@@ -411,8 +402,8 @@ def run_biot_savart(args, dev):
                     flush, stream)
     plan.sync()
     per_step = 3 * n_elem * (p + 1) ** 2
-    # one recursion (the segment chain's two levels) and three weighted sums (one FMA per column each)
-    flops = (point_level_order_flops(p) + level_flops(p) + 3 * 2 * (p + 1) ** 2) * n_elem
+    # one unit-density pass, and three real multiples of complex values a direction and degree
+    madds = (direction_madds("segment", "const", ("single",), p) + 18 * (p + 1) ** 2) * n_elem
     _emit({"metric": "vector line-density Q2X element-moments/s (three components, Eq. st3)",
            "value": per_step / (ms_q2x * 1e-3), "unit": "element-moments/s", "n_gpus": 1, "steps": args.steps,
            "warmup": args.warmup, "ms_per_step": ms_q2x, "higher_is_better": True, "dtype": "f64",
@@ -420,9 +411,7 @@ def run_biot_savart(args, dev):
            "config": {"workload": "the mixed ball's %d filament segments with vortex currents along them, %d "
                                   "adaptive leaves, p=12 (one recursion pass for the three components)" % (n_elem,
                                                                                            m["leaf_c"].shape[1])},
-           "roofline": {"bound": "alu", "achieved": flops / (ms_q2x * 1e-3) / 1e12,
-                        "peak": PEAKS["fp64"] / 1e12, "unit": "TFLOP/s",
-                        "frac": flops / (ms_q2x * 1e-3) / PEAKS["fp64"]},
+           "roofline": _integer_roofline(madds, ms_q2x),
            "curl_evaluation": {"targets": n_tgt, "ms": ms_curl, "value": n_tgt / (ms_curl * 1e-3),
                                "unit": "H evaluations/s (root expansion, p=12, radius 2)"}})
 
@@ -478,17 +467,12 @@ def run_leaf_reduce(args, dev):
            "errors_vs_oracle": {"max_abs_vs_sequential_sum": err, "sampled_leaves": 20}})
 
 
-# FP64 operations per (target, triangle) pair as the near-field kernel
-# evaluates the closed form from a precomputed face frame: frame coordinates
-# and height (about 20), three vertex distances (9), three edges of about 17
-# (edge coordinates, the log's argument), the solid angle's denominator (13),
-# the sums (2), and each of the 3 sqrt, 3 divisions, 3 log1p and 1 atan2
-# counted as one
-NEARFIELD_OPS_PER_PAIR = 20 + 9 + 3 * 17 + 13 + 2 + 3 + 3 + 3 + 1
-# FP64 flops per pair ncu counted as executed (2 x DFMA + DADD + DMUL thread
-# instructions, library sequences of sqrt, division, log1p and atan2 included):
-# (2 x 92.31 + 33.24 + 37.07) per elapsed cycle x 59.66 M cycles / 39.54 M pairs
-NEARFIELD_EXECUTED_FLOPS_PER_PAIR = (2 * 92.309745 + 33.237194 + 37.074234) * 59656234.0 / 39541618
+# FP64 instructions per (target, triangle) pair left beside the integer ones
+# (square roots, logarithms, arctangents and quotients are integer) where every
+# edge is far from the target: frame coordinates and height 12, offsets and
+# distances 10, edges 13, the solid angle 9, the rest 3; near edges add five to
+# eight each
+NEARFIELD_FP64_PER_PAIR = 47
 
 
 def run_nearfield(args, dev):
@@ -524,21 +508,15 @@ def run_nearfield(args, dev):
     lists = [range(off[leaf_of[t]], off[leaf_of[t] + 1]) for t in pick]
     ref = onf.potentials("triangle", vx, idx, sig, tgt[:, pick], lists)
     err = float(np.max(np.abs(got[pick] - ref)) / np.max(np.abs(ref)))
-    ops = NEARFIELD_OPS_PER_PAIR * pairs
+    ops = float(NEARFIELD_FP64_PER_PAIR) * pairs
     _emit({"metric": "near-field element potentials/s (exact triangle integrals, Sec. 4.1)",
            "value": pairs / (ms * 1e-3), "unit": "target-element pairs/s", "n_gpus": 1, "steps": args.steps,
            "warmup": args.warmup, "ms_per_step": ms, "higher_is_better": True, "dtype": "f64", "data": "synthetic",
            "config": {"workload": "collocation at the centroids of the level-7 sphere's %d triangles, each against "
                                   "every triangle of its depth-5 leaf: %d pairs, single layer" % (n_elem, pairs)},
-           "roofline": {"bound": "alu", "achieved": ops / (ms * 1e-3) / 1e12, "peak": PEAKS["fp64"] / 1e12,
-                        "unit": "TFLOP/s", "frac": ops / (ms * 1e-3) / PEAKS["fp64"],
-                        "ops_per_pair": NEARFIELD_OPS_PER_PAIR,
-                        "note": "sqrt, division, log and atan2 count as one operation each: a lower bound",
-                        "executed": {"flops_per_pair": NEARFIELD_EXECUTED_FLOPS_PER_PAIR,
-                                     "frac": NEARFIELD_EXECUTED_FLOPS_PER_PAIR * pairs / (ms * 1e-3)
-                                     / PEAKS["fp64"],
-                                     "source": "ncu DFMA/DADD/DMUL counts of one capture of this "
-                                               "kernel on this workload"}},
+           "roofline": {"bound": "fp64 instructions", "achieved": ops / (ms * 1e-3) / 1e12,
+                        "peak": PEAKS["fp64"] / 2 / 1e12, "unit": "Tinstr/s",
+                        "frac": ops / (ms * 1e-3) / (PEAKS["fp64"] / 2), "fp64_per_pair": NEARFIELD_FP64_PER_PAIR},
            "errors_vs_oracle": {"graded_quadrature": err, "sampled_targets": len(pick)}})
 
 
@@ -556,6 +534,7 @@ def run(args):
     from bench import measure_alu_peaks
     pk = measure_alu_peaks(dev, 0.5)
     PEAKS["fp64"] = pk["dfma"]["tflops"] * 1e12
+    PEAKS["imad"] = pk["imad"]["tmadds"] * 1e12
     PEAKS["fp32"] = max(pk["ffma"]["tflops"], pk["ffma2"]["tflops"]) * 1e12
     PEAKS["measured"] = pk
     {"icosphere-L3": run_icosphere_l3, "upward": run_upward,

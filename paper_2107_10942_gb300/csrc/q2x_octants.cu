@@ -15,7 +15,7 @@
 // l = 2 mod 4, while entry (m, j) holds orders m - j and m + j only.
 //
 // Bound: the FP64 pipe (a warp's FP64 instruction holds it for 80 cycles), so
-// the count decides.  At p = 12 a parent costs 5,700 multiply-adds and up to
+// the count decides.  At p = 12 a parent costs 6,500 multiply-adds and up to
 // 24 x 169 additions of W (absent children skip theirs: some 8 on a surface);
 // a child by the general contraction costs 33,000.  The terms are cut into one
 // run of equal length a thread, entries in a transposed list, so no lane
