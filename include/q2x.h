@@ -335,11 +335,13 @@ int64_t q2x_octant_table(int p, int norm, double h, int64_t n_dst, void* table, 
  * where x, y, z of src centre - dst centre are -h, else +h).  table (device)
  * is the one for this p, norm, h and n_dst; another p, norm or split sets
  * bit 1 of the device error word and writes nothing.  An octant outside 0..7
- * sets bit 1 and that source adds zero.  Sources of one destination are
+ * sets bit 1 and that source adds zero.  delta: NULL, or double[3 * n_src] SoA,
+ * what each source's shift has beyond +-h (at most 2^-32 h: it is applied to
+ * first order).  Sources of one destination are
  * combined before they are translated: one translation a destination. */
 q2x_status q2x_translate_octants(q2x_plan_t plan, int p, int64_t n_src, const double* src_coef, const void* table,
-                                 const int32_t* oct, int64_t n_dst, const int64_t* dst_off, double* dst_coef,
-                                 int accumulate);
+                                 const int32_t* oct, const double* delta, int64_t n_dst, const int64_t* dst_off,
+                                 double* dst_coef, int accumulate);
 
 /* Far-field evaluation (the M2P step fed by the leaf or box coefficients):
  * out[t] (+)= sum over the expansions e listed for target t of

@@ -329,10 +329,12 @@ class Plan:
         p = self.p_max if p is None else int(p)
         return OctantTable(p, self.norm, int(n_dst), octant_table_host(p, self.norm, h, n_dst).to(device))
 
-    def translate_octants(self, src_coef, table, octant, dst_off, dst_coef=None, accumulate=False, p=None):
+    def translate_octants(self, src_coef, table, octant, dst_off, dst_coef=None, accumulate=False, p=None,
+                          delta=None):
         """translate() for one octree level, children to parents: source s lies
         in octant[s] (bits 0, 1, 2: x, y, z of its shift negative) of its
-        destination (q2x_translate_octants)."""
+        destination; delta (3, n_src) is what its shift has beyond +-h, if it
+        has (q2x_translate_octants)."""
         p = self.p_max if p is None else int(p)
         nc = n_coef(p)
         _need(src_coef, torch.float64, "src_coef")
@@ -340,6 +342,7 @@ class Plan:
             raise ValueError("src_coef must be (n_src, (p+1)^2)")
         n_src = src_coef.shape[0]
         _need(octant, torch.int32, "octant", (n_src,))
+        _need(delta, torch.float64, "delta", (3, n_src))
         _need(dst_off, torch.int64, "dst_off")
         n_dst = dst_off.shape[0] - 1
         if dst_coef is None:
@@ -349,7 +352,8 @@ class Plan:
         _need(dst_coef, torch.float64, "dst_coef", (n_dst, nc))
         if (table.p, table.norm, table.n_dst) != (p, self.norm, n_dst):
             raise ValueError("table is not the one of this p, norm and number of destinations")
-        check(lib().q2x_translate_octants(self._h, p, n_src, _ptr(src_coef), _ptr(table.data), _ptr(octant), n_dst,
+        check(lib().q2x_translate_octants(self._h, p, n_src, _ptr(src_coef), _ptr(table.data), _ptr(octant),
+                                          _ptr(delta), n_dst,
                                           _ptr(dst_off), _ptr(dst_coef), int(bool(accumulate))), self._h)
         return dst_coef
 

@@ -111,14 +111,14 @@ class Upward:
         # computed once for the tree (q2x_translation_rows) instead of once
         # per translation and pass
         self.rt = []
-        # per level (table, octants): where every shift is (+-h, +-h, +-h) up
-        # to the rounding of the centres, the level's children are combined
+        # per level (table, octants, rests): where every shift is (+-h, +-h,
+        # +-h) up to the rounding of the centres (the rests, or None if there is
+        # none), the level's children are combined
         # first and translated once a parent (q2x_translate_octants); leaves
         # centred elsewhere in their boxes keep one translation a child
         # (a pass over 3,592 leaves in five levels at p = 12: 69 us, child by
         # child 214 us)
         self.octants = []
-        reach = max(abs(lo), abs(lo + size), size)
         src_c_h = lc[:, deep]
         for lv in self.levels:
             off = torch.from_numpy(lv["dst_off"]).to(device)
@@ -130,10 +130,13 @@ class Upward:
             rt = plan.translation_rows(torch.from_numpy(np.ascontiguousarray(t_tab.T)).to(device), self.p)
             self.rt.append((rt, torch.from_numpy(t_idx.reshape(-1).astype(np.int32)).to(device)))
             h = size / (1 << (self.max_depth - len(self.octants) + 1))
-            if np.abs(np.abs(t) - h).max(initial=0.0) <= 8 * np.finfo(np.float64).eps * reach:
+            delta = t - np.where(t < 0, -h, h)
+            most = np.abs(delta).max(initial=0.0)
+            if most <= h * 2.0 ** -32:
                 octant = ((t < 0) * np.array([[1], [2], [4]])).sum(axis=0).astype(np.int32)
+                rest = torch.from_numpy(np.ascontiguousarray(delta)).to(device) if most > 0.0 else None
                 self.octants.append((plan.octant_table(h, lv["c"].shape[1], self.p, device),
-                                     torch.from_numpy(octant).to(device)))
+                                     torch.from_numpy(octant).to(device), rest))
             else:
                 self.octants.append(None)
             # the boxes of this depth as the next level's sources, gathered
@@ -194,7 +197,8 @@ class Upward:
         outs = []
         for (off, c, out, gidx, nodes_c), (rt, t_idx), octants in zip(self.dev, self.rt, self.octants):
             if precomputed_shifts and octants is not None:
-                self.plan.translate_octants(src, *octants, off, dst_coef=out, p=self.p)
+                table, octant, rest = octants
+                self.plan.translate_octants(src, table, octant, off, dst_coef=out, p=self.p, delta=rest)
             elif precomputed_shifts:
                 self.plan.translate_rt(src, rt, t_idx, off, dst_coef=out, p=self.p)
             else:

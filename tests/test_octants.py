@@ -140,3 +140,58 @@ def test_against_translate(p, n_dst, norm):
     assert torch.equal(got, want)
     with pytest.raises(ValueError):
         plan.translate_octants(dev(src), plan.octant_table(h, n_dst + 1), dev(oct_), dev(off))
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("norm", ["coeff", "moment"])
+@pytest.mark.parametrize("p", [0, 1, 2, 12, 20])
+def test_rounded_centres(p, norm):
+    """Shifts that differ from +-h by up to 1e-10 h: as accurate as with their
+    own shifts (the second order, 190 x 1e-20, is far below the tolerance), and
+    1e-10 n off, so beyond it, without the rest."""
+    import torch
+
+    import paper_2107_10942_gb300 as q2x
+    rng = np.random.default_rng(p)
+    h, nc, n_dst = 0.21, (p + 1) ** 2, 30
+    oct_ = np.tile(np.arange(8), n_dst).astype(np.int32)
+    off = np.arange(0, 8 * n_dst + 1, 8).astype(np.int64)
+    sign = np.where((oct_[None, :] >> np.arange(3)[:, None]) & 1, -h, h)
+    delta = h * 1e-10 * rng.uniform(-1, 1, sign.shape)
+    src_c = sign + delta
+    delta = src_c - sign
+    n = np.array([k for k in range(p + 1) for _ in range(2 * k + 1)])
+    scale = h ** n / np.array([float(math.factorial(k)) for k in n])
+    src = rng.standard_normal((len(oct_), nc)) * scale
+    dev = lambda a: torch.from_numpy(np.ascontiguousarray(a)).cuda()  # noqa: E731
+    plan = q2x.Plan(p, norm=norm)
+    table = plan.octant_table(h, n_dst)
+    want = plan.translate(dev(src), dev(src_c), dev(off), dev(np.zeros((3, n_dst)))).cpu().numpy()
+    top = np.abs(want / scale).max(axis=1, keepdims=True)
+    for rest in (dev(delta), None):
+        got = plan.translate_octants(dev(src), table, dev(oct_), dev(off), delta=rest).cpu().numpy()
+        ok = np.abs(got - want) / scale <= 1e-13 * top
+        assert ok.all() if rest is not None or p == 0 else not ok.all()
+    assert plan.device_errors() == 0
+
+
+@pytest.mark.gpu
+def test_upward_in_any_cube():
+    """A cube whose centres are rounded: the pass as with each child's own shift."""
+    import torch
+
+    import paper_2107_10942_gb300 as q2x
+    from paper_2107_10942_gb300.upward import Upward
+    p, depth, lo, size = 8, 6, -1.1, 2.3
+    rng = np.random.default_rng(2)
+    ijk = np.unique(rng.integers(0, 1 << depth, (500, 3)), axis=0)
+    leaf_c = (lo + (ijk.T + 0.5) * (size / (1 << depth)))
+    n = np.array([k for k in range(p + 1) for _ in range(2 * k + 1)])
+    h = size / (2 << depth)
+    coef = torch.from_numpy(rng.standard_normal((len(ijk), (p + 1) ** 2)) * h ** n).cuda()
+    up = Upward(q2x.Plan(p), leaf_c, lo, size, depth, device="cuda")
+    assert any(o is not None and o[2] is not None for o in up.octants)
+    one = [x.clone() for x in up.run(coef, precomputed_shifts=False)]
+    for k, (a, b) in enumerate(zip(up.run(coef), one)):
+        s = (h * 2.0 ** (k + 1)) ** n
+        assert float(((a - b).cpu().abs() / torch.from_numpy(s)).max()) <= 1e-13 * float((b.cpu().abs() / torch.from_numpy(s)).max())
