@@ -21,7 +21,7 @@
 // Bound: the FP64 pipe (a warp's FP64 instruction holds it for 80 cycles), so
 // the count decides.  At p = 12 a parent costs 6,500 multiply-adds and up to
 // 24 x 169 additions of W (absent children skip theirs: some 8 on a surface);
-// a child by the general contraction costs 33,000.  The terms are cut into one
+// a child by the general contraction costs 12,000.  The terms are cut into one
 // run of equal length a thread, entries in a transposed list, so no lane
 // waits; a run's share of an entry goes to a slot in shared memory, and one
 // thread an entry adds its slots in order (deterministic).
