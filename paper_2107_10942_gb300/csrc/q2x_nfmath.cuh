@@ -166,7 +166,10 @@ NF_SLOW double nf_slow_atan2(double a, double b) { return atan2(a, b); }
 
 // sqrt of x >= 0.  x = X 2^-62 4^k, X in [2^62, 2^64); g0 = sqrt(X) from an
 // FP32 reciprocal root, then two corrections E / (2 g) with the exact
-// remainder E, each adding some 22 bits.
+// remainder E, each adding some 22 bits: the root is known to a few units of
+// 2^-64, and whether it lies above the midpoint 2 r + 1 of its two neighbours r
+// and r + 1 (at 2^53) is decided by the exact sign of m 2^(54 + odd) - (2 r + 1)^2,
+// which is far below 2^63 here and never zero.
 NF_FN double nf_sqrt(double x)
 {
     const nf_u64 b = nf_bits(x);
@@ -184,8 +187,9 @@ NF_FN double nf_sqrt(double x)
     const nf_i64 E1 = (nf_i64)(((nf_u64)E << 31) - (nf_u64)g * (nf_u64)d - (nf_u64)(nf_ws(dh, dh) >> 1));
     const nf_i64 d2 = nf_ws((int)(E1 >> 24), (int)Y) >> 37;
     const nf_u64 G = ((nf_u64)g << 32) + (nf_u64)(d + d2);
-    const nf_u64 r = (G >> 11) + ((G >> 10) & 1);
-    return nf_double(((nf_u64)(k + 1022) << 52) + r);
+    const nf_u64 r = G >> 11, mid = 2 * r + 1;
+    const nf_i64 above = (nf_i64)((m << (54 + odd)) - mid * mid);  // modulo 2^64
+    return nf_double(((nf_u64)(k + 1022) << 52) + r + (above > 0 ? 1u : 0u));
 }
 
 // -------------------------------------------------------------- quotient
