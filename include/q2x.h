@@ -55,6 +55,12 @@
  *    Q2X_ERR_DEVICE_INPUT and clears it.  Invalid elements contribute zero.
  *  - No CPU fallback: without a usable CUDA device every call fails with
  *    Q2X_ERR_CUDA.  No exception crosses the ABI.
+ *  - Stream capture: a captured call uses memory of its plan, which stays
+ *    valid until q2x_plan_destroy also when later calls need more of it
+ *    (far-field calls have scratch of their own per captured call).  Launches of
+ *    one graph, and of graphs captured on one plan and the plan's own calls,
+ *    share that memory unless they are far-field calls: order them on a stream
+ *    or by events.
  *  - Thread safety: a plan may be used by one host thread at a time; distinct
  *    plans are independent.
  */

@@ -95,18 +95,51 @@ namespace {
 
 size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
+// whether the plan's stream is being captured
+bool capturing(q2x_plan_t plan)
+{
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(plan->stream, &cap) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return cap != cudaStreamCaptureStatusNone;
+}
+
+// a buffer to hold until the plan goes
+bool keep_buffer(q2x_plan_t plan, void* p, size_t bytes)
+{
+    try {
+        plan->ws_kept.emplace_back(p, bytes);
+    } catch (...) {
+        return false;
+    }
+    return true;
+}
+
 // grow the workspace to at least `bytes` (synchronises the plan's stream
-// before releasing the old buffer)
+// before releasing the old buffer).  A buffer that a captured graph uses is
+// not released before the plan: the next one is at least twice its size, so
+// that the kept ones together stay below the one in use.
 q2x_status ensure_ws(q2x_plan_t plan, size_t bytes)
 {
-    if (bytes <= plan->ws_bytes) return Q2X_OK;
+    if (bytes <= plan->ws_bytes) {
+        if (!plan->ws_captured) plan->ws_captured = capturing(plan);
+        return Q2X_OK;
+    }
     cudaError_t e;
     if (plan->ws) {
         e = cudaStreamSynchronize(plan->stream);
         if (e != cudaSuccess) return cuda_fail(plan, e, "cudaStreamSynchronize");
-        cudaFree(plan->ws);
+        if (plan->ws_captured) {
+            if (!keep_buffer(plan, plan->ws, plan->ws_bytes)) return fail(plan, Q2X_ERR_OOM, "no host memory");
+            bytes = std::max(bytes, 2 * plan->ws_bytes);
+        } else {
+            cudaFree(plan->ws);
+        }
         plan->ws = nullptr;
         plan->ws_bytes = 0;
+        plan->ws_captured = false;
     }
     bytes = align_up(std::max<size_t>(bytes, 1 << 20), 1 << 20);
     e = cudaMalloc(&plan->ws, bytes);
@@ -115,6 +148,7 @@ q2x_status ensure_ws(q2x_plan_t plan, size_t bytes)
         return fail(plan, Q2X_ERR_OOM, "workspace allocation of %zu bytes failed", bytes);
     }
     plan->ws_bytes = bytes;
+    plan->ws_captured = capturing(plan);  // (a relaxed capture may allocate)
     return Q2X_OK;
 }
 
@@ -600,6 +634,101 @@ q2x_status q2x_plan_workspace(q2x_plan_t plan, size_t bytes)
     return ensure_ws(plan, bytes);
 }
 
+static q2x_status plan_scratch(q2x_plan_t plan, size_t bytes, void** out)
+{
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    cudaGraph_t graph = nullptr;
+    if (cudaStreamGetCaptureInfo(plan->stream, &cap, nullptr, &graph) != cudaSuccess) {
+        cudaGetLastError();  // (the legacy stream beside another stream's capture: the launch will say so)
+        return Q2X_OK;
+    }
+    if (cap == cudaStreamCaptureStatusActive) {
+        // a buffer no graph holds any more, or a new one (cudaMalloc is no
+        // stream operation, but the capture modes forbid it unless relaxed)
+        q2x_graph_scratch s;
+        for (size_t i = 0; i < plan->far_graphs.size(); ++i) {
+            if (!plan->far_graphs[i].dropped->load() || plan->far_graphs[i].bytes < bytes) continue;
+            s = plan->far_graphs[i];
+            plan->far_graphs.erase(plan->far_graphs.begin() + (long)i);
+            break;
+        }
+        cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+        if (cudaThreadExchangeStreamCaptureMode(&mode) != cudaSuccess) return Q2X_OK;
+        if (!s.p) {
+            for (size_t i = plan->far_graphs.size(); i-- > 0;)  // too small for this call: given back
+                if (plan->far_graphs[i].dropped->load()) {
+                    cudaFree(plan->far_graphs[i].p);
+                    plan->far_graphs.erase(plan->far_graphs.begin() + (long)i);
+                }
+            if (cudaMalloc(&s.p, bytes) != cudaSuccess) {
+                cudaGetLastError();
+                s.p = nullptr;
+            }
+            s.bytes = bytes;
+        }
+        cudaThreadExchangeStreamCaptureMode(&mode);
+        if (!s.p) return Q2X_OK;
+        s.dropped = std::make_shared<std::atomic<bool>>(false);
+        auto* held = new std::shared_ptr<std::atomic<bool>>(s.dropped);
+        cudaUserObject_t obj = nullptr;
+        cudaError_t e = cudaUserObjectCreate(
+            &obj, held,
+            [](void* h) {
+                auto* d = static_cast<std::shared_ptr<std::atomic<bool>>*>(h);
+                (*d)->store(true);
+                delete d;
+            },
+            1, cudaUserObjectNoDestructorSync);
+        if (e != cudaSuccess) {
+            cudaGetLastError();
+            delete held;
+            s.dropped->store(true);
+        } else if (cudaGraphRetainUserObject(graph, obj, 1, cudaGraphUserObjectMove) != cudaSuccess) {
+            cudaGetLastError();
+            cudaUserObjectRelease(obj, 1);
+            e = cudaErrorUnknown;
+        }
+        plan->far_graphs.push_back(s);
+        if (e == cudaSuccess) *out = s.p;
+        return Q2X_OK;
+    }
+    if (cap != cudaStreamCaptureStatusNone) return Q2X_OK;
+    if (plan->far && plan->far_stream != plan->stream) {
+        cudaError_t e = cudaStreamWaitEvent(plan->stream, plan->far_left, 0);
+        if (e != cudaSuccess) return q2x_cuda_fail(plan, e, "cudaStreamWaitEvent");
+    }
+    if (bytes > plan->far_bytes) {
+        if (plan->far) {
+            cudaError_t e = cudaStreamSynchronize(plan->stream);  // (waits for the other stream's calls too)
+            if (e != cudaSuccess) return q2x_cuda_fail(plan, e, "cudaStreamSynchronize");
+            cudaFree(plan->far);
+            plan->far = nullptr;
+            plan->far_bytes = 0;
+        }
+        bytes = align_up(bytes, 1 << 20);
+        if (cudaMalloc(&plan->far, bytes) != cudaSuccess) {
+            cudaGetLastError();
+            plan->far = nullptr;
+            return Q2X_OK;
+        }
+        plan->far_bytes = bytes;
+    }
+    plan->far_stream = plan->stream;
+    *out = plan->far;
+    return Q2X_OK;
+}
+
+q2x_status q2x_plan_scratch(q2x_plan_t plan, size_t bytes, void** out)
+{
+    *out = nullptr;
+    try {
+        return plan_scratch(plan, bytes, out);
+    } catch (...) {  // no host memory
+        *out = nullptr;
+        return Q2X_OK;
+    }
+}
+
 q2x_status q2x_galerkin_directions(q2x_plan_t plan, int64_t n_elem, int64_t n_vert, const double* vxyz,
                                    const int32_t* idx, const double* sigma, int64_t n_leaves, const int64_t* leaf_off,
                                    const double* leaf_c, int layer, const double* w, double* out, bool* taken)
@@ -694,6 +823,10 @@ q2x_status q2x_plan_destroy(q2x_plan_t plan)
     cudaSetDevice(plan->device);
     cudaStreamSynchronize(plan->stream);
     if (plan->ws) cudaFree(plan->ws);
+    for (auto& k : plan->ws_kept) cudaFree(k.first);
+    if (plan->far) cudaFree(plan->far);
+    for (auto& g : plan->far_graphs) cudaFree(g.p);
+    if (plan->far_left) cudaEventDestroy(plan->far_left);
     if (plan->d_err) cudaFree(plan->d_err);
     for (cudaEvent_t ev : plan->ev_pool) cudaEventDestroy(ev);
     for (auto& pr : plan->ev_pending) {
@@ -708,7 +841,21 @@ q2x_status q2x_plan_destroy(q2x_plan_t plan)
 q2x_status q2x_plan_set_stream(q2x_plan_t plan, void* cuda_stream)
 {
     if (!plan) return Q2X_ERR_ARG;
-    plan->stream = static_cast<cudaStream_t>(cuda_stream);
+    const cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
+    if (plan->far && plan->stream == plan->far_stream && st != plan->stream) {
+        // the next call that uses the far-field scratch waits for those so far
+        cudaSetDevice(plan->device);
+        cudaError_t e = capturing(plan) ? cudaErrorStreamCaptureUnsupported : cudaSuccess;
+        if (e == cudaSuccess && !plan->far_left) e = cudaEventCreateWithFlags(&plan->far_left, cudaEventDisableTiming);
+        if (e == cudaSuccess) e = cudaEventRecord(plan->far_left, plan->stream);
+        if (e != cudaSuccess) {  // no order to be had: the buffer stays with that stream's calls
+            cudaGetLastError();
+            keep_buffer(plan, plan->far, plan->far_bytes);
+            plan->far = nullptr;
+            plan->far_bytes = 0;
+        }
+    }
+    plan->stream = st;
     return Q2X_OK;
 }
 
@@ -795,7 +942,14 @@ q2x_status q2x_reserve(q2x_plan_t plan, int64_t n_elem, int64_t n_leaves)
     return ensure_ws(plan, bytes);
 }
 
-int64_t q2x_workspace_bytes(q2x_plan_t plan) { return plan ? (int64_t)plan->ws_bytes : -1; }
+int64_t q2x_workspace_bytes(q2x_plan_t plan)
+{
+    if (!plan) return -1;
+    size_t b = plan->ws_bytes + plan->far_bytes;
+    for (auto& k : plan->ws_kept) b += k.second;
+    for (auto& g : plan->far_graphs) b += g.bytes;
+    return (int64_t)b;
+}
 
 q2x_status q2x_segments(q2x_plan_t plan, int64_t n_elem, int64_t n_vert, const double* vxyz,
                         const int32_t* idx, const double* sigma, int64_t n_leaves,

@@ -87,26 +87,17 @@ __global__ void q2x_evaluate_curl_kernel(const EvalArgs a)
 // takes 56 us against 33 at 16,384 targets, 62 against 107 at 65,536, 339
 // against 1,382 at 2^20 (p = 6: 36 against 42, p = 2: 29 against 18 at 65,536);
 // the curl, whose general form is a long FP64 chain, 175 us against 261 at
-// 2,048 targets already.  The workspace stays below 2 GiB and, under stream
-// capture, has to be there.
-static bool take_directions(q2x_plan_t plan, int p, int comps, int64_t n_exp, int64_t n_tgt, q2x_status* st)
+// 2,048 targets already.  The scratch stays below 2 GiB; *ws receives it, NULL
+// where the general path has to run.
+static q2x_status take_directions(q2x_plan_t plan, int p, int comps, int64_t n_exp, int64_t n_tgt, void** ws)
 {
-    *st = Q2X_OK;
+    *ws = nullptr;
     const int64_t entries = (int64_t)(p + 1) * (p + 2) / 2;
-    if (p < 2 || n_exp <= 0 || n_exp > 0x7fffffffLL || n_tgt / 8 < n_exp) return false;
-    if (n_tgt < (comps == 1 ? 3000000 : 180000) / entries) return false;
+    if (p < 2 || n_exp <= 0 || n_exp > 0x7fffffffLL || n_tgt / 8 < n_exp) return Q2X_OK;
+    if (n_tgt < (comps == 1 ? 3000000 : 180000) / entries) return Q2X_OK;
     const size_t bytes = q2x::far_workspace(p, comps, n_exp);
-    if (bytes > ((size_t)2 << 30)) return false;
-    if (bytes > plan->ws_bytes) {
-        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-        if (cudaStreamIsCapturing(plan->stream, &cap) != cudaSuccess) {
-            cudaGetLastError();
-            return false;
-        }
-        if (cap != cudaStreamCaptureStatusNone) return false;
-    }
-    *st = q2x_plan_workspace(plan, bytes);
-    return *st == Q2X_OK;
+    if (bytes > ((size_t)2 << 30)) return Q2X_OK;
+    return q2x_plan_scratch(plan, bytes, ws);
 }
 
 extern "C" q2x_status q2x_evaluate_curl(q2x_plan_t plan, int p, int64_t n_exp, const double* coef3,
@@ -138,14 +129,15 @@ extern "C" q2x_status q2x_evaluate_curl(q2x_plan_t plan, int p, int64_t n_exp, c
     a.exp_idx = exp_idx;
     a.out = out3;
     a.err = plan->d_err;
-    q2x_status st;
-    if (take_directions(plan, p, 3, n_exp, n_tgt, &st)) {
-        e = q2x::far_run(a, 3, plan->ws, plan->stream);
+    void* ws;
+    q2x_status st = take_directions(plan, p, 3, n_exp, n_tgt, &ws);
+    if (st != Q2X_OK) return st;
+    if (ws) {
+        e = q2x::far_run(a, 3, ws, plan->stream);
         if (e != cudaSuccess) return q2x_cuda_fail(plan, e, "far-field direction kernels");
         plan->launches += 3;
         return Q2X_OK;
     }
-    if (st != Q2X_OK) return st;
     q2x::q2x_evaluate_curl_kernel<<<(unsigned)((n_tgt + 127) / 128), 128, 0, plan->stream>>>(a);
     e = cudaGetLastError();
     if (e != cudaSuccess) return q2x_cuda_fail(plan, e, "q2x_evaluate_curl_kernel launch");
@@ -180,14 +172,15 @@ extern "C" q2x_status q2x_evaluate(q2x_plan_t plan, int p, int64_t n_exp, const 
     a.exp_idx = exp_idx;
     a.out = out;
     a.err = plan->d_err;
-    q2x_status st;
-    if (take_directions(plan, p, 1, n_exp, n_tgt, &st)) {
-        e = q2x::far_run(a, 1, plan->ws, plan->stream);
+    void* ws;
+    q2x_status st = take_directions(plan, p, 1, n_exp, n_tgt, &ws);
+    if (st != Q2X_OK) return st;
+    if (ws) {
+        e = q2x::far_run(a, 1, ws, plan->stream);
         if (e != cudaSuccess) return q2x_cuda_fail(plan, e, "far-field direction kernels");
         plan->launches += 3;
         return Q2X_OK;
     }
-    if (st != Q2X_OK) return st;
     const int64_t grid = (n_tgt + 127) / 128;
     q2x::q2x_evaluate_kernel<<<(unsigned)grid, 128, 0, plan->stream>>>(a);
     e = cudaGetLastError();
