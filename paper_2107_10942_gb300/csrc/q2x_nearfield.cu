@@ -88,7 +88,7 @@ __device__ __forceinline__ void line_factors(double sm, double sp, double Rm, do
     const bool behind = (nf_bits(sg) >> 63) != 0;
     const double a = behind ? Rp : Rm;
     const nf_u64 s = behind ? nf_bits(sp) ^ (1ull << 63) : nf_bits(sm);
-    const bool ahead = (s >> 63) == 0;
+    const bool ahead = s <= 1ull << 63;  // s >= 0, a negative zero too (an end of the piece: e = 0, not 0 / 0)
     const double w = a + nf_double(s & 0x7fffffffffffffffull);
     b = Sg + nf_double(nf_bits(sg) & 0x7fffffffffffffffull);
     c = ahead ? 1.0 : w;
