@@ -206,7 +206,7 @@ __device__ __forceinline__ void face_potential(const Face* __restrict__ Fp, V3 r
 {
     const double J = __ldg(&Fp->J);
     single = solid = h_out = 0.0;
-    if (nf_bits(J) == 0) return;  // J > 0 or exactly zero
+    if (nf_bits(J) - 1 >= 0x7ff0000000000000ull) return;  // zero or NaN (J is never negative)
     const V3 x1{__ldg(&Fp->x1[0]), __ldg(&Fp->x1[1]), __ldg(&Fp->x1[2])};
     const V3 d = sub(r, x1);
     const double rx = d.x * __ldg(&Fp->u[0]) + d.y * __ldg(&Fp->u[1]) + d.z * __ldg(&Fp->u[2]);
@@ -290,7 +290,10 @@ __global__ void __launch_bounds__(128) q2x_nearfield_kernel(const NearArgs a, co
         j0 = j1 = 0;
     }
     const V3 r{__ldg(a.tgt + t), __ldg(a.tgt + a.n_tgt + t), __ldg(a.tgt + 2 * a.n_tgt + t)};
-    const double tol_r = NF_SNAP * (fabs(r.x) + fabs(r.y) + fabs(r.z));
+    // (a NaN bound would lie above every distance's bits, NaN ones too, where
+    // the comparison of a NaN has to fail: the target's own NaN stays in the result)
+    double tol_r = NF_SNAP * (fabs(r.x) + fabs(r.y) + fabs(r.z));
+    if (tol_r != tol_r) tol_r = 0.0;
     double acc = 0.0;
 #pragma unroll 1
     for (int64_t j = j0; j < j1; ++j) {
