@@ -290,16 +290,25 @@ __global__ void leaf_reduce_weighted_kernel(const double* __restrict__ elem, int
 // Elements per leaf tile of the FP32-mixed single-layer path.
 constexpr int64_t kLeafTileElems = 256;
 
+// Calls whose tile list and partial rows would need more than this run the
+// element kernel.
+constexpr size_t kLeafTileWsMax = (size_t)8 << 30;
+
 // workspace of the leaf-tile paths (after the per-leaf scales): the tile list,
-// the scans, and the partial rows of leaves of several tiles
-size_t leaf_tile_ws_bytes(int64_t n_elem, int64_t n_leaves, int np, int64_t T, int layers = 1)
+// the scans, and the partial rows of leaves of several tiles; full: tiles that
+// the elements would fill
+size_t leaf_tile_ws_bytes_of(int64_t full, int64_t n_leaves, int np, int layers)
 {
     const int64_t nb = q2x::leaf_tile_blocks(n_leaves);
-    const int64_t mt = q2x::leaf_tile_max_tiles(n_leaves, n_elem, T);
-    const int64_t ms = q2x::leaf_tile_max_slots(n_elem, T);
+    const int64_t mt = q2x::leaf_tile_max_tiles(n_leaves, full, 1);
+    const int64_t ms = q2x::leaf_tile_max_slots(full, 1);
     return align_up(sizeof(q2x::BatchTile) * (size_t)mt, 256) + 2 * align_up(sizeof(int64_t) * (size_t)n_leaves, 256) +
            2 * align_up(sizeof(int64_t) * (size_t)nb, 256) + align_up(sizeof(int64_t) * (size_t)(n_leaves + 1), 256) +
            256 + 256 + layers * align_up(sizeof(double) * (size_t)ms * np, 256);
+}
+size_t leaf_tile_ws_bytes(int64_t n_elem, int64_t n_leaves, int np, int64_t T, int layers = 1)
+{
+    return leaf_tile_ws_bytes_of((n_elem + T - 1) / T, n_leaves, np, layers);
 }
 
 // the arrays of that workspace, from p on
@@ -460,7 +469,7 @@ q2x_status run_elements(q2x_plan_t plan, int kind, int dens, int64_t n_elem, int
     // 8 GiB the element kernel, whose workspace is per warp range, runs)
     const bool tiles = prec == 1 && leaf_off && !vec && coef0 && !(kind == q2x::KIND_TRI && coef1) &&
                        n_leaves < ((int64_t)1 << 31) &&
-                       leaf_tile_ws_bytes(n_elem, n_leaves, np, kLeafTileElems) <= ((size_t)8 << 30);
+                       leaf_tile_ws_bytes(n_elem, n_leaves, np, kLeafTileElems) <= kLeafTileWsMax;
     // FP64 in leaf mode: the same tile list through the direction kernels
     // (q2x_dir.cuh), within the same workspace bound
     const bool dirs = prec == 0 && leaf_off && n_leaves < ((int64_t)1 << 31);
@@ -474,7 +483,7 @@ q2x_status run_elements(q2x_plan_t plan, int kind, int dens, int64_t n_elem, int
         if (e != cudaSuccess) return cuda_fail(plan, e, "direction tables");
         dir_bytes = leaf_tile_ws_bytes(n_elem, n_leaves, np, shape.T, dir_layers);
     }
-    if (dirs && dir_bytes <= ((size_t)8 << 30)) {
+    if (dirs && dir_bytes <= kLeafTileWsMax) {
         q2x_status st = ensure_ws(plan, dir_bytes);
         if (st != Q2X_OK) return st;
         return run_directions(plan, da, combo, shape, n_elem, n_vert, vxyz, idx, sigma, n_leaves, leaf_off,
@@ -736,7 +745,7 @@ q2x_status q2x_galerkin_directions(q2x_plan_t plan, int64_t n_elem, int64_t n_ve
     const int p = plan->p_max, np = (p + 1) * (p + 1);
     const q2x::DirShape shape = q2x::dir_shape(p, 1, n_elem, n_leaves, plan->num_sms);
     const size_t bytes = leaf_tile_ws_bytes(n_elem, n_leaves, np, shape.T, 0);
-    *taken = n_leaves < ((int64_t)1 << 31) && bytes <= ((size_t)8 << 30);
+    *taken = n_leaves < ((int64_t)1 << 31) && bytes <= kLeafTileWsMax;
     if (!*taken) return Q2X_OK;
     q2x_status st = ensure_ws(plan, bytes);
     if (st != Q2X_OK) return st;
@@ -929,14 +938,14 @@ q2x_status q2x_reserve(q2x_plan_t plan, int64_t n_elem, int64_t n_leaves)
     // worst case: one range per 32 elements; FP64 partials in both precisions
     const int64_t n_ranges = (n_elem + 31) / 32;
     const size_t elem = align_up(sizeof(double) * (size_t)n_ranges * 2 * 3 * np, 256);
+    // the tile lists of this size and of every smaller one, whose tiles may be
+    // smaller (q2x::dir_most_tiles); larger lists are not used
     size_t tile = 0;
     if (plan->prec == 1)
         tile = leaf_tile_ws_bytes(n_elem, n_leaves, np, kLeafTileElems);
     else
-        for (int layers = 1; layers <= 3; ++layers)
-            tile = std::max(tile, leaf_tile_ws_bytes(n_elem, n_leaves, np,
-                                                     q2x::dir_shape(plan->p_max, layers, n_elem, n_leaves, plan->num_sms).T, layers));
-    if (tile > ((size_t)8 << 30)) tile = 0;  // such calls run the element kernel
+        tile = leaf_tile_ws_bytes_of(q2x::dir_most_tiles(plan->p_max, n_elem, plan->num_sms), n_leaves, np, 3);
+    tile = std::min(tile, kLeafTileWsMax);
     const size_t bytes = std::max(elem, tile) + align_up(sizeof(double) * (size_t)n_leaves, 256) +
                          align_up(sizeof(int) * (size_t)n_leaves, 256);
     return ensure_ws(plan, bytes);

@@ -85,6 +85,12 @@ DirShape dir_shape(int p, int layers, int64_t n_elem, int64_t n_leaves, int num_
     return s;
 }
 
+int64_t dir_most_tiles(int p, int64_t n_elem, int num_sms)
+{
+    const int64_t T = dir_tile_elems(p, 64);
+    return std::min(n_elem, std::max((n_elem + T - 1) / T, 2 * (int64_t)num_sms));
+}
+
 cudaError_t dir_tables(int p, DirTables* t)
 {
     void *vec, *inv, *eighth, *pw, *col;

@@ -905,6 +905,10 @@ struct DirShape {
     int cls, nt, T;
 };
 DirShape dir_shape(int p, int layers, int64_t n_elem, int64_t n_leaves, int num_sms);
+// The most tiles dir_shape can cut up to n_elem elements into, leaves apart:
+// full tiles of the smallest CTA, or, where they are spread over the SMs, tiles
+// of at least n_elem / num_sms (rounded down, so up to two an SM).
+int64_t dir_most_tiles(int p, int64_t n_elem, int num_sms);
 // Elements a tile may hold: eight a group (the number format's head room), at
 // most one a thread (the frames).
 inline int dir_tile_elems(int p, int nt)

@@ -146,3 +146,21 @@ def test_captured_elements_survive_growth(q2x):
     plan.sync()
     assert torch.equal(out, ref)
     del junk
+
+
+@pytest.mark.parametrize("p,n_res,l_res,calls", [(20, 433, 64, [(311, 64), (433, 1), (152, 64)]),
+                                                (12, 9000, 300, [(9000, 300), (4000, 300), (1300, 2), (310, 300)])])
+def test_reserve_covers_smaller_calls(q2x, p, n_res, l_res, calls):
+    # smaller calls may take smaller tiles and so more of them
+    from paper_2107_10942_gb300.q2x import problem_to_device
+    plan = q2x.Plan(p)
+    plan.reserve(n_res, l_res)
+    held = plan.workspace_bytes()
+    for n, nl in calls:
+        sizes = [n // nl + (1 if k < n % nl else 0) for k in range(nl)]
+        prob = random_problem("triangle", sizes, seed=n, p=p)
+        d = problem_to_device({k: v for k, v in prob.items() if hasattr(v, "shape")})
+        plan.triangles(d["vxyz"], d["idx"], d["sigma"], d["leaf_off"], d["leaf_c"], single=True, double=True)
+        plan.triangles(d["vxyz"], d["idx"], d["sigma"], d["leaf_off"], d["leaf_c"])
+        plan.sync()
+        assert plan.workspace_bytes() == held, (n, nl)
