@@ -10,31 +10,34 @@ namespace q2x {
 
 namespace {
 
+// The limit on dynamic shared memory belongs to the function, for all plans and
+// threads of the process, so it is the same at every set: the opt-in 227 KB
+// less room for the static arrays.
+constexpr int kDirSmemMax = 225 * 1024;
+
 template <int KIND, int DENS, int OUTS, int MAX_NT>
-cudaError_t dir_attr(int p, int nt, int T, size_t* smem)
+cudaError_t dir_attr()
 {
-    *smem = DirCfg<KIND, DENS, OUTS>::smem(p, T, nt);
     return cudaFuncSetAttribute(q2x_dir_kernel<KIND, DENS, OUTS, MAX_NT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)*smem);
+                                kDirSmemMax);
 }
 
 template <int KIND, int DENS, int OUTS, int MAX_NT>
 cudaError_t dir_launch(const DirArgs& a, int nt, int T, int grid, cudaStream_t st)
 {
-    size_t smem;
-    cudaError_t e = dir_attr<KIND, DENS, OUTS, MAX_NT>(a.p_max, nt, T, &smem);
+    const cudaError_t e = dir_attr<KIND, DENS, OUTS, MAX_NT>();
     if (e != cudaSuccess) return e;
-    q2x_dir_kernel<KIND, DENS, OUTS, MAX_NT><<<grid, nt, smem, st>>>(a, T);
+    q2x_dir_kernel<KIND, DENS, OUTS, MAX_NT><<<grid, nt, DirCfg<KIND, DENS, OUTS>::smem(a.p_max, T, nt), st>>>(a, T);
     return cudaGetLastError();
 }
 
 template <int KIND, int DENS, int OUTS, int MAX_NT>
 cudaError_t dir_occupancy(int* blocks, int p, int nt, int T)
 {
-    size_t smem;
-    cudaError_t e = dir_attr<KIND, DENS, OUTS, MAX_NT>(p, nt, T, &smem);
+    const cudaError_t e = dir_attr<KIND, DENS, OUTS, MAX_NT>();
     if (e != cudaSuccess) return e;
-    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks, q2x_dir_kernel<KIND, DENS, OUTS, MAX_NT>, nt, smem);
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks, q2x_dir_kernel<KIND, DENS, OUTS, MAX_NT>, nt,
+                                                         DirCfg<KIND, DENS, OUTS>::smem(p, T, nt));
 }
 
 #define Q2X_DIR_FNS(K, D, O, M) {&dir_launch<K, D, O, M>, &dir_occupancy<K, D, O, M>}
