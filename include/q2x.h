@@ -100,7 +100,12 @@ typedef struct q2x_plan_s* q2x_plan_t;
 
 /* Create a plan for degrees up to p_max (0..Q2X_P_MAX) in the given norm and
  * precision, bound to a CUDA stream (cudaStream_t; NULL = legacy default
- * stream) on the current device.  Q2X_FP64 runs the whole recursion in FP64.
+ * stream) on the current device.  Q2X_FP64 gives results to FP64 accuracy:
+ * per-element rows (leaf_off NULL) and batches by recursions in FP64, leaf sums
+ * in 62-bit fixed point with a power of two for every element, level and degree
+ * (the error of a degree of a leaf sum is a few units of 2^-53 of the sum of the
+ * elements' magnitudes at that degree, as from FP64 sums, however uneven the
+ * elements are).
  * Q2X_FP32_MIXED runs it in FP32 in a per-leaf scaled local frame; the
  * translation to the leaf centre keeps FP64 accuracy (exact double -> float
  * splitting), per-leaf sums are FP32 with compensated combination of partial
@@ -364,8 +369,10 @@ q2x_status q2x_translate_octants(q2x_plan_t plan, int p, int64_t n_src, const do
  *            and is skipped, a bad range (or a non-empty list with exp_idx
  *            NULL) sets bit 8 and the target gets 0
  *   out      double[n_tgt] (device), overwritten or added to (accumulate = 1)
- * FP64 arithmetic in both precisions of the plan; S_n^m by the
- * associated-Legendre recurrences in Cartesian form (Eqs. (bas1)-(bas2)). */
+ * FP64 accuracy in both precisions of the plan: S_n^m by the
+ * associated-Legendre recurrences in Cartesian form (Eqs. (bas1)-(bas2)) in FP64
+ * or, with many targets an expansion, by directions in 62-bit fixed point where
+ * a target's terms fill it (see q2x_farfield.cu). */
 q2x_status q2x_evaluate(q2x_plan_t plan, int p, int64_t n_exp, const double* coef, const double* exp_c,
                         int64_t n_tgt, const double* tgt, const int64_t* tgt_off, const int64_t* exp_idx,
                         double* out, int accumulate);
@@ -379,8 +386,9 @@ q2x_status q2x_evaluate(q2x_plan_t plan, int p, int64_t n_exp, const double* coe
  *   coef3   double[3 * n_exp * (p+1)^2]: component-major [3][n_exp][np] (device)
  *   out3    double[3 * n_tgt] SoA (device)
  * Other arguments as q2x_evaluate.  The gradients of S_n^m are carried
- * through the same recurrences in forward mode (no derivative tables).  COEFF
- * norm only (Q2X_ERR_UNSUPPORTED otherwise).  FP64. */
+ * through the same recurrences in forward mode (no derivative tables), or by
+ * the directions' derivatives.  COEFF norm only (Q2X_ERR_UNSUPPORTED
+ * otherwise).  FP64 accuracy. */
 q2x_status q2x_evaluate_curl(q2x_plan_t plan, int p, int64_t n_exp, const double* coef3, const double* exp_c,
                              int64_t n_tgt, const double* tgt, const int64_t* tgt_off, const int64_t* exp_idx,
                              double* out3, int accumulate);
@@ -430,7 +438,9 @@ q2x_status q2x_nearfield(q2x_plan_t plan, int kind, int layer, int64_t n_elem, i
  *   (sigma required: the per-element weights)
  *   w    double[n_leaves * (p_max+1)^2] (device)
  *   out  double[n_elem] (device), overwritten
- * FP64 arithmetic in both precisions of the plan; deterministic. */
+ * FP64 accuracy in both precisions of the plan (62-bit fixed point in every
+ * element's own scale: an error of a few units of 2^-53 of the element's own
+ * terms); deterministic. */
 q2x_status q2x_galerkin_triangles(q2x_plan_t plan, int64_t n_elem, int64_t n_vert, const double* vxyz,
                                   const int32_t* idx, const double* sigma, int64_t n_leaves,
                                   const int64_t* leaf_off, const double* leaf_c, const double* leaf_rho,
@@ -450,10 +460,10 @@ q2x_status q2x_leaf_reduce(q2x_plan_t plan, int64_t n_elem, int p, const double*
  * (component j's block at coef3 + j * n_leaves * (p_max+1)^2), otherwise the
  * arguments of q2x_segments (leaf_off required).  The moments are geometric
  * and each component multiplies them, so the recursion runs once per
- * element, with unit density: each round's moments are staged once and summed
- * per leaf three times, weighted by the components (one pass of the element
- * kernel; no temporary beyond the plan workspace).  Same results as three
- * q2x_segments calls with the components as densities, up to rounding;
+ * element, with unit density, and its values are summed per leaf three times,
+ * weighted by the components (one pass; no temporary beyond the plan
+ * workspace).  Same results as three q2x_segments calls with the components as
+ * densities, up to rounding, each component relative to its own magnitudes;
  * deterministic.  A non-finite component sets Q2X_DEVERR_NONFINITE and its
  * segment contributes zero. */
 q2x_status q2x_segments_vector(q2x_plan_t plan, int64_t n_elem, int64_t n_vert, const double* vxyz,

@@ -479,7 +479,7 @@ q2x_status run_elements(q2x_plan_t plan, int kind, int dens, int64_t n_elem, int
     size_t dir_bytes = 0;
     if (dirs) {
         da.p_max = plan->p_max;
-        e = q2x::dir_setup(da, kind, dens, shape.nt);
+        e = q2x::dir_setup(da, shape.nt);
         if (e != cudaSuccess) return cuda_fail(plan, e, "direction tables");
         dir_bytes = leaf_tile_ws_bytes(n_elem, n_leaves, np, shape.T, dir_layers);
     }
@@ -751,7 +751,7 @@ q2x_status q2x_galerkin_directions(q2x_plan_t plan, int64_t n_elem, int64_t n_ve
     if (st != Q2X_OK) return st;
     q2x::DirArgs a{};
     a.p_max = p;
-    cudaError_t e = q2x::dir_setup(a, q2x::KIND_TRI, Q2X_DENSITY_CONST, shape.nt);
+    cudaError_t e = q2x::dir_setup(a, shape.nt);
     if (e != cudaSuccess) return cuda_fail(plan, e, "direction tables");
     q2x::LeafTileWork lw;
     leaf_tile_carve(static_cast<unsigned char*>(plan->ws), n_elem, n_leaves, np, shape.T, 0, lw, nullptr);

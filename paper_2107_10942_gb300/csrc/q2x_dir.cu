@@ -58,15 +58,16 @@ const DirFns& dir_fns(int cls, int combo)
 }
 
 // 256 threads where two such CTAs fit an SM's shared memory (p = 16, single
-// layer: 255 of them at work), else the most that do (constant density, both
-// layers, p = 12: 1.76 ms with 192 threads, 2.11 with one CTA of 256); a vector
-// density takes one CTA of 256 as long as that fits (2M segments, p = 12: 4.3
-// ms, 4.7 with two of 160).  Where leaves are small a tile keeps few groups
-// busy and its frames bound it, so more and smaller CTAs overlap better
-// (800,000 triangles, p = 16: 13 a leaf 2.5 ms with 128 threads, 3.3 with 256;
-// 3 a leaf 5.7 with 64, 8.9 with 256; p = 8: 13 a leaf 0.80 with 64, 1.55 with
-// 256; 53 a leaf 256 is ahead at p = 12, 1.12 against 1.18 ms, and 40 tetrahedra a
-// leaf at p = 10, 0.26 against 0.31, but behind at p = 8, 0.70 against 0.56).
+// layer: 255 of them at work), else the most that do (800,000 triangles, 200 a
+// leaf, both layers, p = 12: 1.67 ms with 192 threads, 2.05 with one CTA of 256);
+// a vector density takes one CTA of 256 as long as that fits (2M segments, p =
+// 12: 4.5 ms, two of 160 the same).  Where leaves are small a tile keeps few
+// groups busy and its frames bound it, so more and smaller CTAs overlap better
+// (800,000 triangles, p = 16: 13 a leaf 2.9 ms with 128 threads, 3.9 with 256; 3 a
+// leaf 7.3 with 64, 13.5 with 256; p = 8: 13 a leaf 0.88 with 64, 1.90 with 256).
+// The line for 128: 53 a leaf 1.15 against 1.31 ms at p = 12 and 1.86 against 2.06
+// at p = 16, but 3.08 against 2.86 at p = 20, and 75 a leaf 1.26 against 1.16 at p =
+// 12; 40 tetrahedra a leaf 1.14 against 1.45 at p = 10, 0.81 against 1.12 at p = 8.
 DirShape dir_shape(int p, int layers, int64_t n_elem, int64_t n_leaves, int num_sms)
 {
     const double mean = (double)n_elem / (double)std::max<int64_t>(n_leaves, 1);
@@ -75,7 +76,7 @@ DirShape dir_shape(int p, int layers, int64_t n_elem, int64_t n_leaves, int num_
     auto smem = [&](int nt) { return (size_t)(p + 1) * (16 * layers * nt + 48) + (size_t)nt / (p + 1) * 1024; };
     const size_t most = layers == 3 ? 200 * 1024 : 110 * 1024;
     while (s.nt > 128 && smem(s.nt) > most) s.nt -= 32;
-    if (mean < (p >= 10 ? 32.0 : 96.0) && layers < 3) {
+    if (mean < (p > 16 ? 48.0 : p >= 10 ? 56.0 : 96.0) && layers < 3) {
         s.nt = mean < (p >= 10 ? 5.0 : 20.0) ? 64 : 128;
         s.cls = (p >= 12 && s.nt == 128) ? 0 : 1;
     }
@@ -96,22 +97,18 @@ int64_t dir_most_tiles(int p, int64_t n_elem, int num_sms)
 
 cudaError_t dir_tables(int p, DirTables* t)
 {
-    void *vec, *inv, *eighth, *pw, *col;
+    void *vec, *inv, *col;
     cudaError_t e = cudaGetSymbolAddress(&vec, g_dir_vec);
     if (e == cudaSuccess) e = cudaGetSymbolAddress(&inv, g_dir_inv);
-    if (e == cudaSuccess) e = cudaGetSymbolAddress(&eighth, g_dir_eighth);
-    if (e == cudaSuccess) e = cudaGetSymbolAddress(&pw, g_dir_pow);
     if (e == cudaSuccess) e = cudaGetSymbolAddress(&col, g_dir_col);
     if (e != cudaSuccess) return e;
     t->vec = static_cast<const int2*>(vec) + h_dir_vec_off[p];
     t->inv = static_cast<const int2*>(inv) + h_dir_inv_off[p];
-    t->eighth = static_cast<const int2*>(eighth);
-    t->pw = static_cast<const double*>(pw);
     t->col = static_cast<const double*>(col);
     return cudaSuccess;
 }
 
-cudaError_t dir_setup(DirArgs& a, int kind, int dens, int nt)
+cudaError_t dir_setup(DirArgs& a, int nt)
 {
     const int p = a.p_max;
     DirTables t;
@@ -119,31 +116,10 @@ cudaError_t dir_setup(DirArgs& a, int kind, int dens, int nt)
     if (e != cudaSuccess) return e;
     a.vec = t.vec;
     a.inv = t.inv;
-    a.eighth = t.eighth;
-    a.pw = t.pw;
     a.col = t.col;
     a.J = p + 1;
     a.G = nt / a.J;
-    a.rnd = (long long)((1ull << 63) + (1ull << 31));
-    // Bound of a level's value over the seed's (|u| < 1): the dimension's
-    // binomial, for linear density (n+1)(n+2)(n+3)/2 of a half.  Seeds start at
-    // 2^55 and values stay below 2^59, so that eight elements' sum fits 62
-    // bits: before the degrees where the bound passes 2^4, 2^7, .. every value
-    // is divided by 2^3 (the low degrees keep more bits than the highest needs).
-    auto bound = [&](int n) {
-        double b = n + 1;
-        if (kind >= KIND_TRI) b *= (n + 2) / 2.0;
-        if (kind == KIND_TET) b *= (n + 3) / 3.0;
-        if (dens == DENS_LINEAR) b = std::max(b, b * (n + 3) / 2.0);
-        return b;
-    };
-    a.seed_bits = 55;
-    double most = 16.0;
-    for (int v = 0; v < 4; ++v, most *= 1 << DIR_EVENT) {
-        int n = 1;
-        while (n <= p && bound(n) <= most) ++n;
-        a.event[v] = n <= p ? n : 1 << 20;
-    }
+    a.rnd = 1ll << 31;
     return cudaSuccess;
 }
 

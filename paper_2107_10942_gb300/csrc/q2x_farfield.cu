@@ -237,8 +237,8 @@ __device__ __noinline__ void general_gradient(const double* F3, int64_t stride, 
     grad_one(F3, stride, p, x, y, z, g);
 }
 
-// y = rho x / r^2 as three Fx and 1/r; false where the general path applies
-__device__ __forceinline__ bool far_point(const FarMeta& m, int p, const double (&x)[3], double r2, Fx (&y)[3],
+// y = rho x / r^2 at 2^62 and 1/r; false where the general path applies
+__device__ __forceinline__ bool far_point(const FarMeta& m, int p, const double (&x)[3], double r2, long long (&y)[3],
                                           double& ir)
 {
     ir = 1.0 / sqrt(r2);
@@ -250,7 +250,7 @@ __device__ __forceinline__ bool far_point(const FarMeta& m, int p, const double 
     if (!(b > 0.0625f)) return false;
 #pragma unroll
     for (int d = 0; d < 3; ++d)
-        y[d] = fx_split(dir_fixed((unsigned long long)__double_as_longlong(x[d] * s), 1022, 62));
+        y[d] = dir_fixed((unsigned long long)__double_as_longlong(x[d] * s), 1022, 62);
     return true;
 }
 
@@ -259,7 +259,7 @@ __global__ void __launch_bounds__(FAR_NT) far_evaluate_kernel(const FarArgs f)
     const EvalArgs& a = f.ev;
     __shared__ int2 dirs[6 * (Q2X_P_MAX + 1)];
     const int J = f.J, p = a.p;
-    for (int i = threadIdx.x; i < 6 * J; i += FAR_NT) dirs[i] = f.tab.vec[i];
+    dir_load(dirs, f.tab.vec, J);
     __syncthreads();
     const int64_t t = (int64_t)blockIdx.x * FAR_NT + threadIdx.x;
     if (t >= a.n_tgt) return;
@@ -280,7 +280,7 @@ __global__ void __launch_bounds__(FAR_NT) far_evaluate_kernel(const FarArgs f)
         const double r2 = offset_r2(a, t, e, x);
         if (!(r2 > 0.0)) continue;  // at the centre the series does not apply
         const FarMeta& m = f.meta[e];
-        Fx y[3];
+        long long y[3];
         double ir;
         if (!far_point(m, p, x, r2, y, ir)) {
             acc += general_potential(a.coef + e * (int64_t)a.np, p, a.norm, x[0], x[1], x[2]);
@@ -291,23 +291,21 @@ __global__ void __launch_bounds__(FAR_NT) far_evaluate_kernel(const FarArgs f)
 #pragma unroll 1
         for (int j = 0; j < J; ++j, c += p + 1) {
             Fx da[6];
-#pragma unroll
-            for (int d = 0; d < 6; ++d) da[d] = as_fx(dirs[j * 6 + d]);
+            dir_of(dirs, j, da);
             const Mul v = mul_of(dir_dot(da, y, rnd), dir_dot(da + 3, y, rnd));
             longlong2 w = __ldg(c);
             Cx b{w.x, w.y};
-            CxH h = high_of<0>(b);
+            CxH h = high_of(b);
             if (p > 0) {
                 const longlong2* q = c - 1;
 #pragma unroll 4
                 for (int n = p - 1; n > 0; --n, --q) {
                     w = __ldg(q);
                     b = mul_add<true>(v, b, h, Cx{w.x, w.y}, rnd);
-                    h = high_of<1>(b);
+                    h = high_of(b);
                 }
                 // the constant term: its real part alone
-                b.re = mul2<true>(v.rh, v.rl, v.nh, v.nl, (int)b.re, h.rh, (int)b.im, h.ih, __ldg(q).x, rnd) -
-                       dir_bias(1);
+                b.re = mul2<true>(v.rh, v.rl, v.nh, v.nl, (int)b.re, h.rh, (int)b.im, h.ih, __ldg(q).x, rnd);
             }
             sum += b.re;
         }
@@ -324,7 +322,7 @@ __global__ void __launch_bounds__(FAR_NT) far_curl_kernel(const FarArgs f)
     const EvalArgs& a = f.ev;
     __shared__ int2 dirs[6 * (Q2X_P_MAX + 1)];
     const int J = f.J, p = a.p;
-    for (int i = threadIdx.x; i < 6 * J; i += FAR_NT) dirs[i] = f.tab.vec[i];
+    dir_load(dirs, f.tab.vec, J);
     __syncthreads();
     const int64_t t = (int64_t)blockIdx.x * FAR_NT + threadIdx.x;
     if (t >= a.n_tgt) return;
@@ -345,7 +343,7 @@ __global__ void __launch_bounds__(FAR_NT) far_curl_kernel(const FarArgs f)
         const double r2 = offset_r2(a, t, e, x);
         if (!(r2 > 0.0)) continue;
         const FarMeta& m = f.meta[e];
-        Fx y[3];
+        long long y[3];
         double ir;
         double g[3][3] = {{0.0, 0.0, 0.0}, {0.0, 0.0, 0.0}, {0.0, 0.0, 0.0}};  // g[k][d] = d A_k / d x_d
         if (!far_point(m, p, x, r2, y, ir)) {
@@ -359,28 +357,26 @@ __global__ void __launch_bounds__(FAR_NT) far_curl_kernel(const FarArgs f)
 #pragma unroll 1
                 for (int j = 0; j < J; ++j, c += p + 1) {
                     Fx da[6];
-#pragma unroll
-                    for (int d = 0; d < 6; ++d) da[d] = as_fx(dirs[j * 6 + d]);
+                    dir_of(dirs, j, da);
                     const Mul v = mul_of(dir_dot(da, y, rnd), dir_dot(da + 3, y, rnd));
                     longlong2 w = __ldg(c);
-                    // b: the polynomial, d: its derivative (both with bias 1)
-                    Cx b{w.x + dir_bias(1), w.y + dir_bias(1)}, d{dir_bias(1), dir_bias(1)};
-                    CxH hb = high_of<1>(b), hd = high_of<1>(d);
+                    // b: the polynomial, d: its derivative
+                    Cx b{w.x, w.y}, d{0, 0};
+                    CxH hb = high_of(b), hd = high_of(d);
                     const longlong2* q = c - 1;
 #pragma unroll 2
                     for (int n = p - 1; n >= 0; --n, --q) {
                         w = __ldg(q);
-                        d = mul_add<true>(v, d, hd, Cx{b.re - dir_bias(1), b.im - dir_bias(1)}, rnd);
-                        hd = high_of<1>(d);
+                        d = mul_add<true>(v, d, hd, b, rnd);
+                        hd = high_of(d);
                         b = mul_add<true>(v, b, hb, Cx{w.x, w.y}, rnd);
-                        hb = high_of<1>(b);
+                        hb = high_of(b);
                     }
-                    val += b.re - dir_bias(1);
+                    val += b.re;
 #pragma unroll
                     for (int i = 0; i < 3; ++i)  // Re(a_i d)
                         der[i] += mul2<false>(da[i].h, da[i].l, -da[3 + i].h, -da[3 + i].l, (int)d.re, hd.rh, (int)d.im,
-                                              hd.ih, 0, rnd) -
-                                  dir_bias(1);
+                                              hd.ih, 0, rnd);
                 }
                 const double L = (double)val * unit;
                 double D[3], dot = 0.0;
@@ -423,7 +419,7 @@ cudaError_t far_run(const EvalArgs& ev, int comps, void* ws, cudaStream_t st)
     if (e != cudaSuccess) return e;
     f.J = ev.p + 1;
     f.comps = comps;
-    f.rnd = (long long)((1ull << 63) + (1ull << 31));
+    f.rnd = 1ll << 31;
     unsigned char* w = static_cast<unsigned char*>(ws);
     f.near = reinterpret_cast<int*>(w);
     w += up(sizeof(int) * (size_t)ev.n_exp);

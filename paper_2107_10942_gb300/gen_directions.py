@@ -115,7 +115,7 @@ def split(v, hi_bits, lo_bits):
     t = (v + (1 << (FRAC - hi_bits - lo_bits - 1))) >> (FRAC - hi_bits - lo_bits)
     h = (t + (1 << (lo_bits - 1))) >> lo_bits
     l = t - (h << lo_bits)
-    assert abs(h) < (1 << 31) and abs(l) <= (1 << 30)
+    assert abs(h) < (1 << 31) and abs(l) < (1 << 30)  # (the kernels double and negate l)
     return h, l
 
 
@@ -146,27 +146,12 @@ def write(path):
         for row in table:
             for v in row:
                 invs += split(v, 30, 28)
-    # 2^(k/8 - 1), k = -7 .. 7, as (h, l) of 62 fractional bits
-    eighth = []
-    for k in range(-7, 8):
-        v = 1 << (8 * FRAC + k + 8 * 2)  # (2^(k/8 + 2) 2^FRAC)^8
-        r = math.isqrt(math.isqrt(math.isqrt(v)))
-        eighth += split(r >> 3, 31, 31)
     with open(path, "w") as f:
         f.write("// Generated by gen_directions.py: constant tables of the direction kernels.\n")
         f.write(_ints("g_dir_vec", vecs) + "\n")
         f.write(_ints("g_dir_inv", invs) + "\n")
-        f.write(_ints("g_dir_eighth", eighth) + "\n")
         f.write("static const int h_dir_vec_off[%d] = {%s};\n" % (P_MAX + 1, ",".join(map(str, vec_off))))
         f.write("static const int h_dir_inv_off[%d] = {%s};\n" % (P_MAX + 1, ",".join(map(str, inv_off))))
-        # 2^(-k n / 8), k = -7 .. 7, n = 0 .. 23
-        pw = []
-        for k in range(-7, 8):
-            for n in range(24):
-                e, r = divmod(-k * n, 8)
-                root = math.isqrt(math.isqrt(math.isqrt(1 << (8 * FRAC + r))))
-                pw.append((root / (1 << FRAC)) * 2.0 ** e)
-        f.write("static __device__ const double g_dir_pow[%d] = {%s};\n" % (len(pw), ",".join(float(v).hex() for v in pw)))
         # per column and hat depth d: n! / (sqrt((n+m)! (n-m)!) (n+d)!), and the same / 4 pi
         pi = 0
         x5, x239 = 5, 239  # Machin: pi = 16 atan(1/5) - 4 atan(1/239)
