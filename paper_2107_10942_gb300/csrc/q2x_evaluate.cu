@@ -82,18 +82,22 @@ __global__ void q2x_evaluate_curl_kernel(const EvalArgs a)
 }  // namespace q2x
 
 // Whether a call takes the direction path (q2x_farfield.cu).  Its three
-// launches and the preparation of an expansion (about eight targets' worth)
-// have to be made up for: with one expansion a target the potential at p = 12
-// takes 56 us against 33 at 16,384 targets, 62 against 107 at 65,536, 339
-// against 1,382 at 2^20 (p = 6: 36 against 42, p = 2: 29 against 18 at 65,536);
-// the curl, whose general form is a long FP64 chain, 175 us against 261 at
-// 2,048 targets already.  The scratch stays below 2 GiB; *ws receives it, NULL
+// launches and the preparation of the expansions have to be made up for: with
+// one expansion the potential at p = 12 takes 56 us against 33 at 16,384 targets,
+// 60 against 107 at 65,536, 327 against 1,382 at 2^20 (p = 6: 36 against 42, p = 2:
+// 29 against 18 at 65,536); the curl, whose general form is a long FP64 chain,
+// 119 us against 173 at 2,200 targets already.  An expansion costs as much as 18 (p =
+// 16) to 45 targets (p = 4) of one list entry; how long the lists are is not known
+// here.  At p = 12 and 65,536 targets 1,000 expansions take 93 us against 107,
+// 2,000 128 against 107 with one entry a target and 371 against 822 with eight
+// (8,000: 343 against 107 and 596 against 822); at p = 4 and 600,000 targets 10,000
+// 243 against 187.  The scratch stays below 2 GiB; *ws receives it, NULL
 // where the general path has to run.
 static q2x_status take_directions(q2x_plan_t plan, int p, int comps, int64_t n_exp, int64_t n_tgt, void** ws)
 {
     *ws = nullptr;
     const int64_t entries = (int64_t)(p + 1) * (p + 2) / 2;
-    if (p < 2 || n_exp <= 0 || n_exp > 0x7fffffffLL || n_tgt / 8 < n_exp) return Q2X_OK;
+    if (p < 2 || n_exp <= 0 || n_exp > 0x7fffffffLL || n_tgt / (p < 8 ? 64 : 32) < n_exp) return Q2X_OK;
     if (n_tgt < (comps == 1 ? 3000000 : 180000) / entries) return Q2X_OK;
     const size_t bytes = q2x::far_workspace(p, comps, n_exp);
     if (bytes > ((size_t)2 << 30)) return Q2X_OK;

@@ -8,17 +8,19 @@
 // of (a_j . y)^n for the null vectors a_j of gen_directions.py: with v = a_j . y
 //     phi(x) = (1/r) sum_j Re sum_n c_{n,j} v^n,
 // one complex Horner step per direction and degree, run in the 64-bit fixed
-// point of q2x_dir.cuh.  y = rho x / r^2 with rho just below the distance of
-// the expansion's nearest target, so |v| < 1; the c_{n,j} are scaled by their
-// own sum, so no partial sum leaves the format.
+// point of q2x_dir.cuh.  y = rho x / r^2 with rho just below the distance that
+// all but a few of the expansion's targets have, so |v| < 1; the c_{n,j} are
+// scaled by the bound of their sums, so no partial sum leaves the format.
 //
-// Three kernels: the nearest distance per expansion; the c_{n,j} of each
-// expansion (one CTA, exact dot products with the left inverse's rows); one
-// thread per target over its list.  The fixed point's error is relative to the
-// terms at the nearest target, so a target where the terms' bound has fallen
-// below a sixteenth of that (far out without a monopole, or beside a target
-// inside the expansion's sphere), and an expansion whose scale leaves FP64,
-// takes the general FP64 evaluation.
+// Three kernels: how often each distance occurs, per expansion, in a sample of
+// the targets; the c_{n,j} of each expansion (one CTA, exact dot products with
+// the left inverse's rows); one thread per target over its list.  The fixed
+// point's error is relative to the terms at rho, so a target where the terms'
+// bound has fallen below a sixteenth of that (far out without a monopole), one
+// nearer than rho, and an expansion whose scale leaves FP64, takes the general
+// FP64 evaluation.  With rho from the nearest target, one close target sent
+// all the others there (2^20 targets at p = 12 1,467 us, now 327; the curl at 2^18
+// 2,900, now 517).
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -32,6 +34,12 @@ namespace {
 
 constexpr int FAR_NT = 128;
 
+// distances are counted in classes of r^2, two an octave, modulo FAR_CLASSES
+// (the largest of a residue stands for it)
+constexpr int FAR_CLASSES = 32;
+constexpr int FAR_SAMPLE = 4096;  // targets an expansion to be counted, on average
+constexpr int FAR_FEW = 1024;     // one in so many targets may be nearer than rho
+
 struct FarMeta {
     double rho;  // 0: not usable
     int scale;   // c = value 2^scale
@@ -43,7 +51,9 @@ struct FarArgs {
     DirTables tab;
     int J, comps;  // 1 potential, 3 curl
     long long rnd;
-    int* near;        // [n_exp] upper words of the smallest r^2
+    int* count;       // [n_exp][FAR_CLASSES]
+    int* cls;         // [n_exp][FAR_CLASSES] the class, upper word of r^2 >> 19
+    int64_t step;     // every step'th warp's targets are counted
     FarMeta* meta;    // [n_exp]
     longlong2* c;     // [comps][n_exp][J][p + 1]
 };
@@ -65,37 +75,44 @@ __device__ __forceinline__ void list_of(const EvalArgs& a, int64_t t, int64_t& j
     if (bad) j0 = j1 = 0;
 }
 
-__global__ void far_near_kernel(const FarArgs f)
+__global__ void far_count_kernel(const FarArgs f)
 {
     const EvalArgs& a = f.ev;
-    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const int64_t warp = (int64_t)blockIdx.x * (FAR_NT / 32) + (threadIdx.x >> 5);
+    const int64_t t = warp * f.step * 32 + (threadIdx.x & 31);
     int64_t j0 = 0, j1 = 0;
     bool bad;
     if (t < a.n_tgt) list_of(a, t, j0, j1, bad);
     for (int64_t j = j0; __any_sync(0xffffffffu, j < j1); ++j) {
         int64_t e = -1;
-        int key = 0x7fffffff;
+        int cls = 0;
         if (j < j1) {
             e = __ldg(a.exp_idx + j);
             if (e >= 0 && e < a.n_exp) {
                 double x[3];
-                const double r2 = offset_r2(a, t, e, x);
-                if (r2 > 0.0) key = hi32(__double_as_longlong(r2));
+                const int key = hi32(__double_as_longlong(offset_r2(a, t, e, x)));
+                cls = key >> 19;
+                if (key < 0x00100000 || key >= 0x7ff00000) e = -1;  // not a normal positive number
             } else {
                 e = -1;
             }
         }
-        // one atomic a warp where the warp shares the expansion, as most do
+        // one atomic a warp and class where the warp shares the expansion, as most do
+        int n = e >= 0 ? 1 : 0;
         const int64_t e0 = __shfl_sync(0xffffffffu, e, 0);
         if (__all_sync(0xffffffffu, e == e0)) {
-            key = __reduce_min_sync(0xffffffffu, key);
-            if ((threadIdx.x & 31) != 0) key = 0x7fffffff;
+            const unsigned same = __match_any_sync(0xffffffffu, cls);
+            n = (threadIdx.x & 31) == __ffs(same) - 1 ? __popc(same) : 0;
         }
-        if (e >= 0 && key < 0x7ff00000 && key < *(volatile int*)(f.near + e)) atomicMin(f.near + e, key);
+        if (e >= 0 && n) {
+            const int64_t at = e * FAR_CLASSES + (cls & (FAR_CLASSES - 1));
+            atomicAdd(f.count + at, n);
+            if (cls > *(volatile int*)(f.cls + at)) atomicMax(f.cls + at, cls);
+        }
     }
 }
 
-// One CTA per (expansion, component): the scaled weights of the packed
+// One CTA per expansion: the scaled weights of the packed
 // columns, degree by degree (a warp each), their exact products with the left
 // inverse, and the common scale.
 __global__ void __launch_bounds__(FAR_NT) far_prepare_kernel(const FarArgs f)
@@ -107,9 +124,24 @@ __global__ void __launch_bounds__(FAR_NT) far_prepare_kernel(const FarArgs f)
     __shared__ int2 s_g[(Q2X_P_MAX + 1) * (Q2X_P_MAX + 1)];
     __shared__ long long s_r[3][(Q2X_P_MAX + 1) * 2 * (Q2X_P_MAX + 1)];
     __shared__ int s_e[3][Q2X_P_MAX + 1];
-    __shared__ double s_sum[3][Q2X_P_MAX + 1];
-    const double rho = __longlong_as_double((long long)f.near[e] << 32);
-    const double rr = (f.near[e] < 0x7ff00000) ? sqrt(rho) * (1.0 - 1e-6) : 0.0;
+    __shared__ double s_top[3][Q2X_P_MAX + 1];
+    // rho: the lower end of the first class at or below which one in FAR_FEW of the
+    // counted targets lies (a warp runs the general path for a single lane of it:
+    // with one in 16, lists of 5 of 64 expansions 1,155 us against 456)
+    __shared__ int s_cls;
+    if (warp == 0) {
+        const int n = f.count[e * FAR_CLASSES + lane], cls = f.cls[e * FAR_CLASSES + lane];
+        int all = 0, upto = 0;
+        for (int o = 0; o < 32; ++o) {
+            const int no = __shfl_sync(0xffffffffu, n, o), co = __shfl_sync(0xffffffffu, cls, o);
+            all += no;
+            if (co <= cls) upto += no;
+        }
+        const int first = __reduce_min_sync(0xffffffffu, n > 0 && FAR_FEW * (int64_t)upto >= all ? cls : 0x7fffffff);
+        if (lane == 0) s_cls = first == 0x7fffffff ? 0 : first;
+    }
+    __syncthreads();
+    const double rr = sqrt(__longlong_as_double((long long)s_cls << 51)) * (1.0 - 1e-6);
     const double inv = rr > 0.0 ? 1.0 / rr : 0.0;
     for (int k3 = 0; k3 < f.comps; ++k3) {
         const double* F = a.coef + ((int64_t)k3 * a.n_exp + e) * np;
@@ -149,7 +181,7 @@ __global__ void __launch_bounds__(FAR_NT) far_prepare_kernel(const FarArgs f)
                 }
             }
             __syncwarp();
-            double sum = 0.0;
+            float most = 0.f;
 #pragma unroll
             for (int c = 0; c < 2; ++c) {
                 const int s = lane + 32 * c;
@@ -164,44 +196,46 @@ __global__ void __launch_bounds__(FAR_NT) far_prepare_kernel(const FarArgs f)
                     }
                     hh += mid >> 28;
                     s_r[k3][n * 2 * J + s] = hh;
-                    sum += fabs((double)hh);
+                    most = fmaxf(most, fabsf((float)hh));
                 }
             }
-            for (int d = 16; d; d >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, d);
+            most = __int_as_float(__reduce_max_sync(0xffffffffu, __float_as_int(most)));
             if (lane == 0) {
                 s_e[k3][n] = ex - 1022 - 58;
-                s_sum[k3][n] = top < 0x7ff00000 ? sum : __longlong_as_double(0x7ff0000000000000ll);
+                // (a direction's two parts together)
+                s_top[k3][n] = top < 0x7ff00000 ? 1.41422 * most : __longlong_as_double(0x7ff0000000000000ll);
             }
             __syncwarp();
         }
         __syncthreads();
     }
-    // the common scale: sum_n (n + 1, for the derivatives) sum_s |c| below 2^59
+    // the common scale: sum_n (n + 1, for the derivatives) max_j |c| below 2^58,
+    // so that the J directions' values add up below 2^63
     __shared__ int s_scale;
     if (threadIdx.x == 0) {
         int most = -100000;  // exponent of the largest degree's sum
         for (int k3 = 0; k3 < f.comps; ++k3)
             for (int n = 0; n <= p; ++n)
-                if (s_sum[k3][n] > 0.0)
-                    most = max(most, s_e[k3][n] + (int)((__double_as_longlong(s_sum[k3][n]) >> 52) & 0x7ff) - 1022);
+                if (s_top[k3][n] > 0.0)
+                    most = max(most, s_e[k3][n] + (int)((__double_as_longlong(s_top[k3][n]) >> 52) & 0x7ff) - 1022);
         double B = 0.0;
         for (int k3 = 0; k3 < f.comps; ++k3) {
             double b = 0.0;
             for (int n = 0; n <= p; ++n)
-                b += (f.comps == 3 ? n + 1.0 : 1.0) * s_sum[k3][n] * pow2d(max(s_e[k3][n] - most, -1000));
+                b += (f.comps == 3 ? n + 1.0 : 1.0) * s_top[k3][n] * pow2d(max(s_e[k3][n] - most, -1000));
             B = fmax(B, b);
         }
         // B 2^most bounds every partial sum
         int scale = 0;
         bool ok = rr > 0.0 && inv < 1e300 && B < 1e300;  // (an infinite weight takes the general path)
-        if (B > 0.0) scale = 59 - (most + (int)((__double_as_longlong(B) >> 52) & 0x7ff) - 1022);
+        if (B > 0.0) scale = 58 - (most + (int)((__double_as_longlong(B) >> 52) & 0x7ff) - 1022);
         if (scale > 1000 || scale < -1000) ok = false;
         FarMeta m;
         m.rho = ok ? rr : 0.0;
         m.scale = scale;
         for (int n = 0; n <= p; ++n) {
             double b = 0.0;
-            for (int k3 = 0; k3 < f.comps; ++k3) b = fmax(b, s_sum[k3][n] * pow2d(max(s_e[k3][n] - most, -1000)));
+            for (int k3 = 0; k3 < f.comps; ++k3) b = fmax(b, s_top[k3][n] * pow2d(max(s_e[k3][n] - most, -1000)));
             m.bound[n] = B > 0.0 ? (float)((f.comps == 3 ? n + 1.0 : 1.0) * b / B) : 0.f;
         }
         if (!(B > 0.0)) m.bound[0] = 1.f;
@@ -407,7 +441,7 @@ size_t up(size_t x) { return (x + 255) / 256 * 256; }
 
 size_t far_workspace(int p, int comps, int64_t n_exp)
 {
-    return up(sizeof(int) * (size_t)n_exp) + up(sizeof(FarMeta) * (size_t)n_exp) +
+    return 2 * up(sizeof(int) * FAR_CLASSES * (size_t)n_exp) + up(sizeof(FarMeta) * (size_t)n_exp) +
            up(sizeof(longlong2) * (size_t)n_exp * comps * (p + 1) * (p + 1));
 }
 
@@ -421,15 +455,19 @@ cudaError_t far_run(const EvalArgs& ev, int comps, void* ws, cudaStream_t st)
     f.comps = comps;
     f.rnd = 1ll << 31;
     unsigned char* w = static_cast<unsigned char*>(ws);
-    f.near = reinterpret_cast<int*>(w);
-    w += up(sizeof(int) * (size_t)ev.n_exp);
+    f.count = reinterpret_cast<int*>(w);
+    w += up(sizeof(int) * FAR_CLASSES * (size_t)ev.n_exp);
+    f.cls = reinterpret_cast<int*>(w);
+    w += up(sizeof(int) * FAR_CLASSES * (size_t)ev.n_exp);
     f.meta = reinterpret_cast<FarMeta*>(w);
     w += up(sizeof(FarMeta) * (size_t)ev.n_exp);
     f.c = reinterpret_cast<longlong2*>(w);
-    e = cudaMemsetAsync(f.near, 0x7f, sizeof(int) * (size_t)ev.n_exp, st);
+    e = cudaMemsetAsync(f.count, 0, 2 * up(sizeof(int) * FAR_CLASSES * (size_t)ev.n_exp), st);  // (and the classes)
     if (e != cudaSuccess) return e;
     const unsigned grid = (unsigned)((ev.n_tgt + FAR_NT - 1) / FAR_NT);
-    far_near_kernel<<<grid, FAR_NT, 0, st>>>(f);
+    f.step = std::max<int64_t>(1, ev.n_tgt / (ev.n_exp * FAR_SAMPLE));
+    const int64_t warps = ((ev.n_tgt + 31) / 32 + f.step - 1) / f.step, per = FAR_NT / 32;
+    far_count_kernel<<<(unsigned)((warps + per - 1) / per), FAR_NT, 0, st>>>(f);
     far_prepare_kernel<<<(unsigned)ev.n_exp, FAR_NT, 0, st>>>(f);
     if (comps == 1)
         far_evaluate_kernel<<<grid, FAR_NT, 0, st>>>(f);
