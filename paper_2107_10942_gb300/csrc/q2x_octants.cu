@@ -290,12 +290,17 @@ static int64_t octant_table(int p, int norm, double h, int64_t n_dst, void* tabl
     };
     std::vector<std::vector<Term>> rows(np);
     std::vector<int> chi(np);
-    for (int i = 0; i < np; ++i) chi[i] = parity_of(entry_of(i));
+    std::vector<Entry> entries(np);
+    for (int i = 0; i < np; ++i) {
+        entries[i] = entry_of(i);
+        chi[i] = parity_of(entries[i]);
+    }
     int64_t total = 0;
     for (int i = 0; i < np; ++i) {
-        const Entry e = entry_of(i);
+        const Entry& e = entries[i];
+        rows[i].reserve((size_t)(e.n + 1) * (e.n + 1));
         for (int j = 0; j < (e.n + 1) * (e.n + 1); ++j) {
-            const Entry f = entry_of(j);
+            const Entry& f = entries[j];
             const int k = e.n - f.n;
             // F^{-f.m} = (-1)^{f.m} conj F^{f.m}
             bool re = false, im = false;

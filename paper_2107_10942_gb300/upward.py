@@ -106,11 +106,10 @@ class Upward:
         self.identity = len(deep) == nl and bool(np.array_equal(deep, np.arange(nl)))
         self.deep_idx = torch.from_numpy(deep).to(device)
         self.dev = []
-        # per level: the distinct shifts t = c_src - c_dst of its translations
-        # (eight on an octree level) and each source's shift, so that R(t) is
-        # computed once for the tree (q2x_translation_rows) instead of once
-        # per translation and pass
-        self.rt = []
+        # per level: each child's shift t = c_src - c_dst, and, where a level takes
+        # them, the distinct ones' rows of R(t), computed once for the tree
+        # (q2x_translation_rows) instead of once per translation and pass
+        self._shifts, self._rows = [], []
         # per level (table, octants, rests): where every shift is (+-h, +-h,
         # +-h) up to the rounding of the centres (the rests, or None if there is
         # none), the level's children are combined
@@ -126,9 +125,8 @@ class Upward:
             out = torch.empty((c.shape[1], nc), dtype=torch.float64, device=device)
             dest = np.repeat(np.arange(lv["c"].shape[1]), np.diff(lv["dst_off"]))
             t = src_c_h - lv["c"][:, dest]
-            t_tab, t_idx = np.unique(t.T, axis=0, return_inverse=True)
-            rt = plan.translation_rows(torch.from_numpy(np.ascontiguousarray(t_tab.T)).to(device), self.p)
-            self.rt.append((rt, torch.from_numpy(t_idx.reshape(-1).astype(np.int32)).to(device)))
+            self._shifts.append(t)
+            self._rows.append(None)
             h = size / (1 << (self.max_depth - len(self.octants) + 1))
             delta = t - np.where(t < 0, -h, h)
             most = np.abs(delta).max(initial=0.0)
@@ -139,6 +137,7 @@ class Upward:
                                      torch.from_numpy(octant).to(device), rest))
             else:
                 self.octants.append(None)
+                self._rows_of(len(self._rows) - 1)
             # the boxes of this depth as the next level's sources, gathered
             # from [internal rows of this level; leaf rows]
             n_int = c.shape[1]
@@ -151,6 +150,21 @@ class Upward:
                 nodes_c = torch.from_numpy(np.ascontiguousarray(allc[:, gidx])).to(device)
                 self.dev.append((off, c, out, torch.from_numpy(gidx).to(device), nodes_c))
                 src_c_h = allc[:, gidx]
+
+    def _rows_of(self, level):
+        """The distinct shifts' rows of a level and each child's index into them."""
+        if self._rows[level] is None:
+            tab, idx = np.unique(self._shifts[level].T, axis=0, return_inverse=True)
+            device = self.leaf_c.device
+            rt = self.plan.translation_rows(torch.from_numpy(np.ascontiguousarray(tab.T)).to(device), self.p)
+            self._rows[level] = (rt, torch.from_numpy(idx.reshape(-1).astype(np.int32)).to(device))
+        return self._rows[level]
+
+    @property
+    def rt(self):
+        """Per level (rows of R(t), index of each child's): of every level, also of
+        those that a pass translates by octants."""
+        return [self._rows_of(i) for i in range(len(self._rows))]
 
     @staticmethod
     def _deepest_rows(lc, lo, size, depth):
@@ -195,11 +209,12 @@ class Upward:
         src = leaf_coef if self.identity else leaf_coef.index_select(0, self.deep_idx)
         src_c = self.leaf_c if self.identity else self.leaf_c.index_select(1, self.deep_idx)
         outs = []
-        for (off, c, out, gidx, nodes_c), (rt, t_idx), octants in zip(self.dev, self.rt, self.octants):
+        for level, ((off, c, out, gidx, nodes_c), octants) in enumerate(zip(self.dev, self.octants)):
             if precomputed_shifts and octants is not None:
                 table, octant, rest = octants
                 self.plan.translate_octants(src, table, octant, off, dst_coef=out, p=self.p, delta=rest)
             elif precomputed_shifts:
+                rt, t_idx = self._rows[level]
                 self.plan.translate_rt(src, rt, t_idx, off, dst_coef=out, p=self.p)
             else:
                 self.plan.translate(src, src_c, off, c, dst_coef=out, p=self.p)
