@@ -338,7 +338,7 @@ void leaf_tile_carve(unsigned char* p, int64_t n_elem, int64_t n_leaves, int np,
 
 // FP64 leaf sums of one element set by the direction kernels
 q2x_status run_directions(q2x_plan_t plan, q2x::DirArgs& a, int combo, const q2x::DirShape& shape,
-                          int64_t n_elem,                          int64_t n_vert, const double* vxyz, const int32_t* idx, const double* sigma,
+                          int64_t n_elem, int64_t n_vert, const double* vxyz, const int32_t* idx, const double* sigma,
                           int64_t n_leaves, const int64_t* leaf_off, const double* leaf_c, const int32_t* leaf_p,
                           double* coef0, double* coef1, int accumulate, const double* wvec, double* coef2)
 {
@@ -830,7 +830,7 @@ q2x_status q2x_plan_destroy(q2x_plan_t plan)
 {
     if (!plan) return Q2X_ERR_ARG;
     cudaSetDevice(plan->device);
-    cudaStreamSynchronize(plan->stream);
+    const q2x_release release(plan->stream);
     if (plan->ws) cudaFree(plan->ws);
     for (auto& k : plan->ws_kept) cudaFree(k.first);
     if (plan->far) cudaFree(plan->far);

@@ -306,7 +306,7 @@ q2x_status q2x_batch_destroy(q2x_batch_t b)
 {
     if (!b) return Q2X_ERR_ARG;
     cudaSetDevice(b->plan->device);
-    cudaStreamSynchronize(b->plan->stream);
+    const q2x_release release(b->plan->stream);
     free_batch(b);
     return Q2X_OK;
 }

@@ -49,6 +49,26 @@ struct q2x_plan_s {
     std::string last_error;
 };
 
+// While memory is given back: the thread may be capturing a graph on a stream
+// of its own (a garbage collector runs when it likes), and neither a wait on the
+// legacy stream nor cudaFree may end that capture.  Waits for the plan's stream
+// where that can be waited for; freeing waits by itself.
+struct q2x_release {
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    explicit q2x_release(cudaStream_t st)
+    {
+        cudaThreadExchangeStreamCaptureMode(&mode);
+        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+        if (cudaStreamIsCapturing(st, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone)
+            cudaStreamSynchronize(st);
+        else
+            cudaGetLastError();
+    }
+    ~q2x_release() { cudaThreadExchangeStreamCaptureMode(&mode); }
+    q2x_release(const q2x_release&) = delete;
+    q2x_release& operator=(const q2x_release&) = delete;
+};
+
 // status helpers shared by the library's translation units
 q2x_status q2x_fail(q2x_plan_t plan, q2x_status st, const char* fmt, ...);
 q2x_status q2x_cuda_fail(q2x_plan_t plan, cudaError_t e, const char* what);
