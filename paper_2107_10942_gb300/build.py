@@ -27,7 +27,7 @@ def _nvcc() -> str:
 
 
 def _flags():
-    return ARCH + ["-O3", "-std=c++17", "-lineinfo", "-Xcompiler", "-fPIC", "-I", os.path.join(ROOT, "include"),
+    return ARCH + ["-O3", "-std=c++17", "-lineinfo", "-Xcompiler", "-fPIC,-ffp-contract=off", "-I", os.path.join(ROOT, "include"),
                    "-I", CSRC, "-I", OUT]
 
 
