@@ -26,8 +26,10 @@
 // large ones beside small ones cost digits, at any degree: per degree, errors
 // against sums in 113 bits are those of the FP64 row kernel or smaller (kinds,
 // degrees to 20, weights up to 1e8 apart; at the top degree of p = 20, in the
-// root of the sum of squares of its terms, 1.6e-16 for segments, 1.8e-16
-// triangles, 2.4e-16 tetrahedra, 1.5e-16 to 7e-16 linear density, the rows 5e-16).
+// root of the sum of squares of its terms, 1.7e-16 for segments, 2.0e-16
+// triangles, 2.6e-16 tetrahedra, the rows 6e-16 to 7e-16; linear density 1.5e-16 to
+// 7e-16, the largest where a tenth of a tile's elements carry the degree, the rows
+// 4e-16 to 5.6e-16).
 //
 // What bounds it: the integer multiplies, 36 per step of the triangle chain, and
 // beside them the shifts and additions of the format.  The level-9 sphere at p =
